@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "driver.h"
+#include "grid_comm.cuh"
 #include "kernels.h"
 
 namespace mmd {
@@ -48,7 +49,20 @@ static bool debug_on() {
   return v;
 }
 
+// How the blocks of one launch on one level's matrix share it (own.cu): every
+// block's first slice, and the rows its entries read (max_rows 0: not listed).
+struct OwnShares {
+  std::vector<int32_t> first;
+  const int32_t* d_first = nullptr;
+  int max_rows = 0, stride = 0;
+  const int32_t *count = nullptr, *list = nullptr;
+  const uint16_t* lcol = nullptr;
+};
+
 struct Workspace {
+  std::map<std::pair<int, int>, OwnShares> shares;  // by (level, grid)
+  int cluster16 = -1;  // a cluster of 16 blocks can run here (-1: not asked yet)
+  unsigned epoch = 0;  // of the last launch with tagged residuals
   std::map<std::string, std::pair<void*, size_t>> bufs;
   int nsm = 0;
   unsigned* bar = nullptr;  // [0] count, [1] gen
@@ -704,6 +718,104 @@ struct Ctx {
     }
   }
 
+  // The phase words and tagged sums of a launch on `grid` blocks (grid_comm.cuh), zeroed on its stream.
+  void comm_words(GridBarrier& b, const std::string& lane, int MT, int grid, cudaStream_t sl) {
+    const size_t cap = sum_words(2 * 4, ws->nsm) * sizeof(ulonglong2) + ws->nsm * sizeof(unsigned);
+    char* w = buf<char>(ws, "comm" + lane, cap);
+    const size_t sb = sum_words(2 * MT, grid) * sizeof(ulonglong2);
+    b.slots = reinterpret_cast<ulonglong2*>(w);
+    b.flags = reinterpret_cast<unsigned*>(w + sb);
+    CK(cudaMemsetAsync(w, 0, sb + grid * sizeof(unsigned), sl));
+  }
+
+  // The shares of a `grid`-block launch on A^(k) and the rows they read, made
+  // at the first solve with that level and grid and kept with the handle's
+  // workspace (4 bytes a listed row, 2 a matrix entry); max_rows 0 where a
+  // block reads more than kNearMax.
+  const OwnShares& own_shares_of(int k, int grid) {
+    const DCSR& A = h->dl[k].A;
+    const int64_t n = h->dl[k].n;
+    OwnShares& sh = ws->shares[{k, grid}];
+    if (!sh.first.empty()) return sh;
+    const std::string t = std::to_string(k) + "_" + std::to_string(grid);
+    std::vector<int32_t> first = own_shares(A.h_sptr.data(), A.nslices, grid);
+    if (near_fits(n)) {
+      sh.stride = (int)std::min<int64_t>(kNearMax, n);
+      int32_t* d = buf<int32_t>(ws, "ow_f" + t, grid + 1);
+      int32_t* cnt = buf<int32_t>(ws, "ow_c" + t, grid);
+      int32_t* list = buf<int32_t>(ws, "ow_l" + t, size_t(grid) * sh.stride);
+      uint16_t* lcol = buf<uint16_t>(ws, "ow_j" + t, A.sell_nnz);
+      CK(cudaMemcpyAsync(d, first.data(), sizeof(int32_t) * (grid + 1), cudaMemcpyHostToDevice, st));
+      CK(launch_near(sell_of(A), n, grid, d, sh.stride, cnt, list, lcol, st));
+      ++S.kernel_launches;
+      std::vector<int32_t> hc(grid);
+      CK(cudaMemcpyAsync(hc.data(), cnt, sizeof(int32_t) * grid, cudaMemcpyDeviceToHost, st));
+      sync();
+      sh.d_first = d;
+      sh.count = cnt;
+      sh.list = list;
+      sh.lcol = lcol;
+      sh.max_rows = *std::max_element(hc.begin(), hc.end());
+      if (sh.max_rows > sh.stride) sh.max_rows = 0;
+    }
+    sh.first.swap(first);
+    return sh;
+  }
+
+  // One right-hand side of FP64 CG on A^(k) on at most `cap` SMs: the launch
+  // of own.cu; false where it does not fit (a block's rows, their neighbours
+  // and five vectors in one SM's shared memory; about 800k rows) and
+  // solve_kernel runs the solve.  One cluster of 16 SMs while the work (FP64
+  // warp instructions of an iteration: a slice's width and six more) is small,
+  // since its sums take 3,500 cycles against 5,000 and more over a grid (64 x
+  // 64 operator, 1.4k instructions: 4.5 us per iteration against 5.1 on 32
+  // blocks; point-cloud graph of 6,000 rows, 7.7k: 11.1 us against 10.2 on
+  // 76); else a block per two slices, up to every SM (graph of 20,000 rows,
+  // 625 slices: 10.9 us on 152 blocks, 11.9 us on 76).
+  bool own_choice(int k, int cap, OwnPlan* plan, int* grid, bool* cluster) {
+    const DCSR& A = h->dl[k].A;
+    if (plain_cg) return false;
+    const double work = A.sell_nnz / 32.0 + 6.0 * A.nslices;
+    const int ranks = (int)std::min<int64_t>(16, A.nslices);
+    *cluster = work <= 4500.0 && cap >= ranks && cluster_ok();
+    *grid = *cluster ? ranks
+                     : (int)std::min<int64_t>(std::min(cap, own_max_grid(ws->nsm)), std::max<int64_t>(16, A.nslices / 2));
+    if (*grid < 1) return false;
+    const OwnShares& sh = own_shares_of(k, *grid);
+    if (!own_plan(A.h_sptr.data(), sh.first.data(), *grid, sh.max_rows, plan)) return false;
+    plan->first = sh.d_first;
+    plan->stride = sh.stride;
+    plan->count = sh.count;
+    plan->list = sh.list;
+    plan->lcol = sh.lcol;
+    return true;
+  }
+
+  bool cluster_ok() {  // sixteen SMs of one GPC
+    if (ws->cluster16 < 0) ws->cluster16 = own_cluster_fits(16) ? 1 : 0;
+    return ws->cluster16 == 1;
+  }
+  bool plain_cg = false;  // solve_kernel for mode 0 too (the autotuner times its grids)
+
+  // One launch of a tile's solve on the caller's stream; own.cu instead of
+  // solve_kernel for one right-hand side of FP64 CG.
+  cudaError_t launch_tile(SolverArgs& a, int k, int MT, int grid) {
+    OwnPlan plan;
+    int g = 0;
+    bool cl = false;
+    if (MT != 1 || a.mode != 0 || a.fp32 || a.df || a.b64 ||
+        !own_choice(k, coop_grid_cap() > 0 ? coop_grid_cap() : ws->nsm, &plan, &g, &cl))
+      return launch_solver(a, MT, grid, st);
+    if (!cl) comm_words(a.bar, "", MT, g, st);
+    const size_t n = (size_t)h->dl[k].n;
+    auto it = ws->bufs.find("own_rt");
+    const bool fresh = it == ws->bufs.end() || it->second.second < n * sizeof(ulonglong2);
+    plan.rt = buf<ulonglong2>(ws, "own_rt", n);
+    if (fresh) CK(cudaMemsetAsync(plan.rt, 0, n * sizeof(ulonglong2), st));  // tag 0: no launch's
+    plan.epoch = ++ws->epoch;
+    return launch_own_cg(a, plan, g, cl, st);
+  }
+
   void solve_raw(int k, int mode, bool fp32, const void* B, void* X, int m, int x0, double tol, int maxit,
                  std::vector<int64_t>* iters, int64_t* inner_total, int* notconv, const double* B64 = nullptr,
                  double* X64 = nullptr, std::vector<int>* conv_out = nullptr) {
@@ -795,7 +907,7 @@ struct Ctx {
         CK(cudaEventCreate(&e1));
         CK(cudaEventRecord(e0, st));
       }
-      CK(launch_solver(a, MT, grid, st));
+      CK(launch_tile(a, k, MT, grid));
       after_launch();
       if (o.profile) CK(cudaEventRecord(e1, st));
       int64_t its[8], inn = 0;
@@ -1488,6 +1600,7 @@ int tune_solver(mmd_handle* h) {
     mmd_eig_opts o;
     mmd_default_eig_opts(&o);
     Ctx c(h, st, o);
+    c.plain_cg = true;
     const int K = (int)h->levels.size();
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));

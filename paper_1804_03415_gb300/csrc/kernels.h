@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "dev_common.cuh"
 
 namespace mmd {
@@ -125,6 +127,35 @@ struct WideArgs {
 };
 int wide_max_grid(int num_sms);
 cudaError_t launch_wide_cg(const WideArgs& a, int grid, cudaStream_t st);
+
+// CG on A, one right-hand side, with every row owned by one thread (own.cu):
+// how one launch lays out its shared memory, and what its blocks read.
+constexpr int kOwnSmem = 224 * 1024;  // dynamic shared memory a block may ask for
+constexpr int kNearMax = 12288;       // rows a block may list
+struct OwnPlan {
+  int slots = 0;                   // 32 x SELL slices of the largest block share
+  int near = 0;                    // room for the listed rows' values
+  int ents = 0;                    // room for staged matrix entries
+  int smem = 0;                    // bytes
+  const int32_t* first = nullptr;  // grid + 1: every block's first slice
+  int stride = 0;                  // of list
+  const int32_t* count = nullptr;  // rows listed by each block
+  const int32_t* list = nullptr;
+  const uint16_t* lcol = nullptr;  // place in its block's list of every entry (SELL order)
+  ulonglong2* rt = nullptr;        // n words {r, tag}; tags of other launches carry another epoch
+  unsigned epoch = 0;              // > 0, another one for every launch that uses rt
+};
+// Shares of equal work: block b takes the slices [first[b], first[b + 1]).
+// sptr: host copy of the slice offsets.
+std::vector<int32_t> own_shares(const int32_t* sptr, int64_t nslices, int grid);
+// near: rows listed by the largest block.  False where the launch does not fit.
+bool own_plan(const int32_t* sptr, const int32_t* first, int grid, int near, OwnPlan* out);
+bool near_fits(int64_t n);
+cudaError_t launch_near(const Sell& A, int64_t n, int grid, const int32_t* first, int stride, int32_t* count,
+                        int32_t* list, uint16_t* lcol, cudaStream_t st);
+int own_max_grid(int num_sms);
+bool own_cluster_fits(int ranks);  // a launch on one cluster of that many blocks
+cudaError_t launch_own_cg(const SolverArgs& a, const OwnPlan& p, int grid, bool cluster, cudaStream_t st);
 
 int solver_threads(int mt);
 int solver_max_grid(int mt, int num_sms);

@@ -41,6 +41,7 @@ struct DCSR {
   int max_row = 0;
   int64_t nslices = 0, sell_nnz = 0;
   int32_t* s_ptr = nullptr;   // nslices + 1, offsets of the slices
+  std::vector<int32_t> h_sptr;  // host copy of s_ptr (the solver's shared-memory plans)
   int32_t* s_len = nullptr;   // nslices, width of each slice
   int32_t* s_row = nullptr;   // 32 * nslices, row of each lane (-1 = padding)
   int32_t* s_col = nullptr;   // sell_nnz
@@ -66,6 +67,7 @@ struct DLevel {
   double* phi_next = nullptr;  // phi^(k+1) per row of this level (device order)
   std::vector<int32_t> perm;   // device position -> natural index (host copy)
   int32_t* d_perm = nullptr;   // same on device
+  bool natural = false;        // perm is the identity
   int32_t* d_iperm = nullptr;  // natural index -> device position
   double eps = 0, delta = 0;   // of P^(k) (k >= 1)
   // V-cycle preconditioner data (present when the handle's mg_ok is set)
