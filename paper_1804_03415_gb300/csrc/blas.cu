@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(BS, MINB)
       for (int u = 0; u < U; ++u)
         if (k + u < len) acc = fma(a[u], xv[u], acc);
     }
-    if (row >= 0) y[row] = acc;
+    if (row >= 0) y[A.out ? A.out[row] : row] = acc;
   }
 }
 

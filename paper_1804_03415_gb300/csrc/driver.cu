@@ -1473,11 +1473,27 @@ int level_spmv(mmd_handle* h, int k, int which, const double* x, double* y, cuda
     mmd_default_eig_opts(&o);
     Ctx c(h, st, o);
     const DLevel& L = h->dl[k];
-    double* a = buf<double>(c.ws, "ls_a", L.n);
-    double* b = buf<double>(c.ws, "ls_b", L.n);
-    k_gather(x, L.n, L.d_perm, L.n, 1, a, L.n, st);
-    c.spmv(k, which, a, b, 1);
-    k_scatter(b, L.n, L.d_perm, L.n, 1, y, L.n, st);
+    const DCSR& A = which ? L.M : L.A;
+    if (A.spmv_variant < 0 || (which == 1 && k == 0)) {
+      double* a = buf<double>(c.ws, "ls_a", L.n);
+      double* b = buf<double>(c.ws, "ls_b", L.n);
+      k_gather(x, L.n, L.d_perm, L.n, 1, a, L.n, st);
+      c.spmv(k, which, a, b, 1);
+      k_scatter(b, L.n, L.d_perm, L.n, 1, y, L.n, st);
+    } else {
+      // the product reads the caller's x where device order is the caller's (and y is another
+      // vector), else a gathered copy, and stores every row at its place in y: one launch or two
+      // instead of three, and no pass over y (128^3 operator: 93 us with the three)
+      Sell S = sell_of(A);
+      if (L.natural && (x + L.n <= y || y + L.n <= x)) {
+        k_spmv(S, x, L.n, y, L.n, 1, st);
+      } else {
+        double* a = buf<double>(c.ws, "ls_a", L.n);
+        k_gather(x, L.n, L.d_perm, L.n, 1, a, L.n, st);
+        S.out = L.d_perm;
+        k_spmv(S, a, L.n, y, L.n, 1, st);
+      }
+    }
     c.sync();
     CK(cudaGetLastError());
   } catch (const CudaFail& f) {

@@ -21,6 +21,7 @@ struct Sell {
   const double* val = nullptr;
   const float* val32 = nullptr;
   const float2* val2 = nullptr;  // double-float copy: value = hi + lo
+  const int32_t* out = nullptr;  // single-column product: entry of y for each row (nullptr: the row itself)
   int variant = -1;  // single-column SpMV kernel picked by k_spmv_autotune (-1: not tuned)
 };
 
