@@ -14,7 +14,6 @@ struct GridBarrier {
   unsigned int* gen;    // unused (kept for layout)
   int* status;          // set to DEV_TIMEOUT when a wait gives up
   long long timeout_ns; // limit of one wait
-  unsigned* flags;      // one phase word per block (grid_comm.cuh; zeroed before each launch)
   ulonglong2* slots;    // tagged partial sums (grid_comm.cuh; zeroed before each launch)
 };
 

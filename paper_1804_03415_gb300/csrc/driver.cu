@@ -650,6 +650,7 @@ struct Ctx {
       a.ir = buf<char>(ws, pre + "ir" + ls, size_t(n) * MT * eb);
       a.ip = buf<char>(ws, pre + "ip" + ls, size_t(n) * MT * eb);
       a.iq = buf<char>(ws, pre + "iq" + ls, size_t(n) * MT * eb);
+      if (mode == 1) a.is = buf<char>(ws, pre + "is" + ls, size_t(n) * MT * eb);
       a.fp32 = fp32 ? 1 : 0;
       a.df = (use_df && mode == 0 && !fp32) ? 1 : 0;
       a.tol = tol;
@@ -668,6 +669,7 @@ struct Ctx {
       if (mode == 3) set_mg(a, mg_deg, mg_only, l);
       if (mode == 4) set_poly(a, poly_deg, l);
       CK(cudaMemsetAsync(bar, 0, sizeof(unsigned) * 64, sl));
+      comm_words(a.bar, ls, MT, grid, sl);
       CK(launch_solver(a, MT, grid, sl));
       after_launch();
     }
@@ -718,14 +720,11 @@ struct Ctx {
     }
   }
 
-  // The phase words and tagged sums of a launch on `grid` blocks (grid_comm.cuh), zeroed on its stream.
+  // The tagged sums of a launch on `grid` blocks (grid_comm.cuh), zeroed on its stream.
   void comm_words(GridBarrier& b, const std::string& lane, int MT, int grid, cudaStream_t sl) {
-    const size_t cap = sum_words(2 * 4, ws->nsm) * sizeof(ulonglong2) + ws->nsm * sizeof(unsigned);
-    char* w = buf<char>(ws, "comm" + lane, cap);
-    const size_t sb = sum_words(2 * MT, grid) * sizeof(ulonglong2);
+    char* w = buf<char>(ws, "comm" + lane, sum_words(2 * 4, ws->nsm) * sizeof(ulonglong2));
     b.slots = reinterpret_cast<ulonglong2*>(w);
-    b.flags = reinterpret_cast<unsigned*>(w + sb);
-    CK(cudaMemsetAsync(w, 0, sb + grid * sizeof(unsigned), sl));
+    CK(cudaMemsetAsync(w, 0, sum_words(2 * MT, grid) * sizeof(ulonglong2), sl));
   }
 
   // The shares of a `grid`-block launch on A^(k) and the rows they read, made
@@ -804,8 +803,10 @@ struct Ctx {
     int g = 0;
     bool cl = false;
     if (MT != 1 || a.mode != 0 || a.fp32 || a.df || a.b64 ||
-        !own_choice(k, coop_grid_cap() > 0 ? coop_grid_cap() : ws->nsm, &plan, &g, &cl))
+        !own_choice(k, coop_grid_cap() > 0 ? coop_grid_cap() : ws->nsm, &plan, &g, &cl)) {
+      comm_words(a.bar, "", MT, grid, st);
       return launch_solver(a, MT, grid, st);
+    }
     if (!cl) comm_words(a.bar, "", MT, g, st);
     const size_t n = (size_t)h->dl[k].n;
     auto it = ws->bufs.find("own_rt");
@@ -845,6 +846,7 @@ struct Ctx {
     void* ir = buf<char>(ws, pre + "ir", size_t(n) * MT * eb);
     void* ip = buf<char>(ws, pre + "ip", size_t(n) * MT * eb);
     void* iq = buf<char>(ws, pre + "iq", size_t(n) * MT * eb);
+    void* is = mode == 1 ? buf<char>(ws, pre + "is", size_t(n) * MT * eb) : nullptr;
     const int ntiles = (m + MT - 1) / MT;
     // several tiles: run them on up to four side streams at once, each grid on
     // a quarter of the SMs (a tile's iteration is latency- and barrier-bound,
@@ -884,6 +886,7 @@ struct Ctx {
       a.ir = ir;
       a.ip = ip;
       a.iq = iq;
+      a.is = is;
       a.fp32 = fp32 ? 1 : 0;
       a.df = (use_df && mode == 0 && !fp32) ? 1 : 0;
       a.tol = tol;

@@ -1,7 +1,7 @@
-// Communication between the blocks of one persistent solve on a cooperative
-// grid: a barrier and a grid-wide sum through tagged words in L2.
+// Sums between the blocks of one persistent solve on a cooperative grid,
+// through tagged words in L2.
 //
-// What bounds them: the round trips to L2 that lie on the critical path
+// What bounds one: the round trips to L2 that lie on the critical path
 // (about 370 cycles each, 840 for a fence behind a store).  An arrival
 // counter followed by a read of the partial sums takes the partials' fence,
 // the atomic add, the poll that sees it and the read of the partials, and the
@@ -25,9 +25,6 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_relaxed(unsigned* p, unsigned v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 // 16-byte {value, tag} words, read and written as one access
 __device__ __forceinline__ void ld_tagged(const ulonglong2* p, unsigned long long& v, unsigned long long& tag) {
   asm volatile(
@@ -42,16 +39,14 @@ __device__ __forceinline__ void st_tagged(ulonglong2* p, unsigned long long v, u
                : "memory");
 }
 
-// One per block: barrier and reduction counters, and a failed wait (sticky).
+// One per block: the number of sums formed, and a failed wait (sticky).
 struct CommSh {
-  unsigned phase;  // barriers passed
-  unsigned nred;   // sums formed
+  unsigned nred;
   int fail;
 };
 
 __device__ __forceinline__ void comm_init(CommSh& cs) {
   if (threadIdx.x == 0) {
-    cs.phase = 0;
     cs.nred = 0;
     cs.fail = 0;
   }
@@ -93,48 +88,6 @@ __device__ __forceinline__ int poll_verdict(const GridBarrier& b, bool ready, un
     }
   }
   return 0;
-}
-
-// Grid-wide barrier of a cooperative launch: what any thread wrote before it
-// is seen by every thread after it.  b.flags: one zeroed word per block.
-__device__ __forceinline__ bool flag_sync(const GridBarrier& b, CommSh& cs) {
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const unsigned G = gridDim.x, lane = threadIdx.x;
-    const unsigned ph = cs.phase + 1;
-    __syncwarp();
-    if (lane == 0) {
-      cs.phase = ph;
-      fence_gpu();
-      st_relaxed(b.flags + blockIdx.x, ph);
-    }
-    const long long t0 = global_ns();
-    unsigned spins = 0;
-    for (unsigned base = 0; base < G; base += 160) {
-      int v;
-      do {
-        unsigned f[5], st = DEV_OK;
-#pragma unroll
-        for (int u = 0; u < 5; ++u) {
-          const unsigned g = base + lane + 32 * u;
-          f[u] = ph;
-          if (g < G) f[u] = ld_relaxed(b.flags + g);
-        }
-        if (lane == 0) st = ld_relaxed((const unsigned*)b.status);
-        bool ready = true;
-#pragma unroll
-        for (int u = 0; u < 5; ++u) ready = ready && (int)(f[u] - ph) >= 0;  // a block may be one phase ahead
-        v = poll_verdict(b, ready, st, spins, t0);
-      } while (v == 0);
-      if (v == 2) {
-        if (lane == 0) cs.fail = 1;
-        break;
-      }
-    }
-    fence_gpu();
-  }
-  __syncthreads();
-  return cs.fail == 0;
 }
 
 // Block-level sum of nv values: part[v * stride + t] is thread t's share,

@@ -78,7 +78,7 @@ struct SolverArgs {
   void* x;
   int x0;
   void *r, *p, *q, *z;
-  void *ir, *ip, *iq;
+  void *ir, *ip, *iq, *is;  // inner CG (mode 1): residual, direction, M r, M p
   int fp32;        // 1: FP32 instance (matrix val32, FP32 vectors)
   int df;          // 1: double-float CG (mode 0): matrix val2, vectors as FP32 pairs, FP64 b and x
   // mode 0 with fp32 = 1 and b64 != NULL: FP32 CG with FP64 reliable updates;

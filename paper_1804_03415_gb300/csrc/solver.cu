@@ -23,11 +23,11 @@
 //
 // Modes
 //   0  CG on A (M = I; the paper's pcg(A, b, -, x0, eps)) in the
-//      Chronopoulos-Gear form: one fused reduction, two barriers/iteration.
+//      Chronopoulos-Gear form: one grid-wide sum and one barrier per iteration.
 //   1  flexible PCG on A with preconditioner M applied by an inner CG;
 //      beta = z+^T (r+ - r) / (r^T z)  (Golub and Ye, 1999), computed as
 //      -alpha z+^T q / (r^T z) since r+ - r = -alpha q.
-//   2  CG on P A P with P = I - Phi Phi^T applied segment by segment.  Since
+//   2  the same on P A P with P = I - Phi Phi^T applied segment by segment.  Since
 //      U of Section 2.3 has orthonormal columns and U U^T = P on each patch,
 //      this is CG on B = U^T A U in the coordinates U g (same iterates); the
 //      solution returned is x = U g.
@@ -36,7 +36,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "dev_common.cuh"
+#include "grid_comm.cuh"
 #include "kernels.h"
 
 namespace mmd {
@@ -55,9 +55,11 @@ constexpr int kMaxThreads = 1024;
 
 template <int MT>
 struct Sh {
+  CommSh comm;
   double quart[2 * MT * 4];  // block reduction: per-warp sums, up to 4 warps per value
+  double sum[2 * MT];        // grid sums of one reduction
   double bn[MT], rz[MT], rr[MT], alpha[MT], val[MT], val2[MT];
-  double irr[MT], irn0[MT], ia[MT];
+  double irr[MT], irn0[MT], ia[MT], iden[MT];
   int act[MT], iact[MT];
   int due[MT], stag[MT];  // reliable updates: replacement due / no progress since the last one
   int ok[MT];             // reliable updates: stopped with the true residual below tol
@@ -81,62 +83,23 @@ __device__ __forceinline__ int64_t share_hi(int64_t n) { return n * (blockIdx.x 
 // shared memory (16 KB for one column, 64 KB for four).
 extern __shared__ double g_part[];
 
-// partial sums red[slot][c][block] -> dst[c] (shared) in every block, and
-// with dst2 also red[slot2][c][block] -> dst2[c]; warp v sums value v, so the
-// values are reduced on different SM sub-partitions
-template <int MT>
-__device__ __forceinline__ void reduce_slot(const double* red, int slot, int m, double* dst, int slot2 = 0,
-                                            double* dst2 = nullptr) {
-  const int G = gridDim.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nv = dst2 ? 2 * m : m;
-  if (w < nv) {
-    const int c = w < m ? w : w - m;
-    const double* p = red + (size_t(w < m ? slot : slot2) * MT + c) * G;
-    double t = 0.0;
-    for (int b = lane; b < G; b += 32) t += p[b];
-    t = warp_sum(t);
-    if (lane == 0) (w < m ? dst : dst2)[c] = t;
-  }
-  __syncthreads();
-}
-
-// Block sums of acc[c], c < m, written to red[slot][c][blockIdx] (and of
-// acc2[c] to red[slot2][c][blockIdx]).  Every thread stores its partials;
-// then wpc warps per value (4 for one or two values, 2 for up to four, else
-// 1) each add a contiguous share with all 32 lanes busy and finish with one
-// shuffle tree.  Consecutive warps sit on different SM sub-partitions, so the
-// FP64 adds of the values proceed in parallel instead of queueing behind one
-// warp.  Fixed order: deterministic.
+// Grid-wide sums of the threads' acc[c] into dst[c], c < m, and of acc2[c]
+// into dst2[c] (both shared), and a full barrier: grid_comm.cuh.
 template <int MT, typename T>
-__device__ __forceinline__ void write_partials(double* red, int slot, int m, const T* acc, Sh<MT>& s,
-                                               const T* acc2 = nullptr, int slot2 = 0) {
+__device__ __forceinline__ bool sum_cols(const GridBarrier& bar, Sh<MT>& s, int m, const T* acc, double* dst,
+                                         const T* acc2 = nullptr, double* dst2 = nullptr) {
   constexpr int NT = threads_for<MT>();
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int nv = acc2 ? 2 * m : m;
+  const int tid = threadIdx.x, nv = acc2 ? 2 * m : m;
 #pragma unroll
   for (int c = 0; c < MT; ++c)
     if (c < m) {
       g_part[c * NT + tid] = (double)acc[c];
       if (acc2) g_part[(m + c) * NT + tid] = (double)acc2[c];
     }
+  if (!grid_sums<true>(bar, s.comm, g_part, NT, nv, 2 * MT, NT, s.quart, s.sum)) return false;
+  if (tid < nv) (tid < m ? dst : dst2)[tid < m ? tid : tid - m] = s.sum[tid];
   __syncthreads();
-  const int wpc = (nv <= 2) ? 4 : (nv <= 4 ? 2 : 1);
-  const int span = NT / wpc;
-  if (w < nv * wpc) {
-    const int v = w / wpc, q = w - v * wpc;
-    const double* p = g_part + v * NT + q * span;
-    double t = 0.0;
-    for (int i = lane; i < span; i += 32) t += p[i];
-    t = warp_sum(t);
-    if (lane == 0) s.quart[v * 4 + q] = t;
-  }
-  __syncthreads();
-  if (tid < nv) {
-    double t = s.quart[tid * 4];
-    for (int q = 1; q < wpc; ++q) t += s.quart[tid * 4 + q];
-    const int c = tid < m ? tid : tid - m;
-    red[(size_t(tid < m ? slot : slot2) * MT + c) * gridDim.x + blockIdx.x] = t;
-  }
+  return true;
 }
 
 // Vector layouts: the caller's b and x are column-major (element (i, c) at
@@ -197,6 +160,60 @@ __device__ __forceinline__ void spmv_cols(const Sell& A, const T* __restrict__ X
       for (int c = 0; c < MT; ++c) xv[c] = msk[c] ? X[jj + c * ld] : T(0);
     }
   };
+  if constexpr (MT == 1) {
+    // A block with few slices (coarse levels: short shares of long rows) would wait for the chains
+    // of load rounds and FMAs of its widest rows on a few warps: a slice's entries are dealt to
+    // several warps and their sums, in shared memory, added in order.
+    const int64_t lo = share_lo(A.nslices);
+    const int nsl = (int)(share_hi(A.nslices) - lo), nw = blockDim.x >> 5, w = threadIdx.x >> 5;
+    int parts = 1;
+    while (parts < 16 && nsl * parts * 2 <= nw) parts *= 2;
+    if (parts > 1) {
+      double* const comb = g_part;  // free between two grid sums
+      const int sl = w / parts, pt = w - sl * parts;
+      if (msk[0] && sl < nsl) {
+        const int32_t base = A.ptr[lo + sl] + lane, len = A.len[lo + sl];
+        const int k1 = len * (pt + 1) / parts;
+        T t = T(0);
+        int k = len * pt / parts;
+        for (; k + 4 <= k1; k += 4) {
+          T av[4], xv[4];
+          int64_t j[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            av[u] = vals[base + (k + u) * 32];
+            j[u] = A.col[base + (k + u) * 32];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) gather(j[u], xv + u);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) t = fma(av[u], xv[u], t);
+        }
+        for (; k < k1; ++k) {
+          T xv;
+          gather(A.col[base + k * 32], &xv);
+          t = fma(vals[base + k * 32], xv, t);
+        }
+        comb[w * 32 + lane] = (double)t;
+      }
+      __syncthreads();
+      if (msk[0] && w < nsl) {
+        const int32_t row = A.row[(lo + w) * 32 + lane];
+        T t = (T)comb[w * parts * 32 + lane];
+        for (int p = 1; p < parts; ++p) t += (T)comb[(w * parts + p) * 32 + lane];
+        if (row >= 0) {
+          Y[row] = t;
+          if (W) {
+            const T wv = W[row];
+            dacc[0] = fma(wv, t, dacc[0]);
+            if (dacc2) dacc2[0] = fma(wv, wv, dacc2[0]);
+          }
+        }
+      }
+      __syncthreads();
+      return;
+    }
+  }
   FOR_BLOCK_SLICES(sl, A.nslices) {
     const int32_t base = A.ptr[sl] + lane, len = A.len[sl];
     const int32_t row = A.row[sl * 32 + lane];
@@ -247,8 +264,9 @@ __device__ __forceinline__ void spmv_cols(const Sell& A, const T* __restrict__ X
 }
 
 template <int MT, typename T>
-__device__ bool inner_cg(const SolverArgs& a, Sh<MT>& s) {
-  // z = M^{-1} r for active columns, CG to relative residual itol (zero start).
+__device__ bool inner_cg_hs(const SolverArgs& a, Sh<MT>& s) {
+  // The same in the Hestenes-Stiefel form, two sums and a barrier per iteration: the FP32
+  // instance, where the other form's delta - beta gamma / alpha' can lose its sign.
   T* const r = (T*)a.r;
   T* const z = (T*)a.z;
   T* const ir = (T*)a.ir;
@@ -280,9 +298,7 @@ __device__ bool inner_cg(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
     spmv_cols<MT, T, true>(a.M, ip, 0, iq, m, s.iact, ip, acc);
-    write_partials<MT, T>(a.red, 2, m, acc, s);
-    if (!grid_sync(a.bar)) return false;
-    reduce_slot<MT>(a.red, 2, m, s.val);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return false;
     if (threadIdx.x < m) s.ia[threadIdx.x] = s.iact[threadIdx.x] ? s.irr[threadIdx.x] / s.val[threadIdx.x] : 0.0;
     __syncthreads();
 #pragma unroll
@@ -297,9 +313,7 @@ __device__ bool inner_cg(const SolverArgs& a, Sh<MT>& s) {
           ir[o] = rv;
           acc[c] = fma(rv, rv, acc[c]);
         }
-    write_partials<MT, T>(a.red, 3, m, acc, s);
-    if (!grid_sync(a.bar)) return false;
-    reduce_slot<MT>(a.red, 3, m, s.val);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.iact[c]) {
@@ -325,6 +339,93 @@ __device__ bool inner_cg(const SolverArgs& a, Sh<MT>& s) {
     *a.in_out += t;
   }
   return true;
+}
+
+template <int MT, typename T>
+__device__ bool inner_cg(const SolverArgs& a, Sh<MT>& s) {
+  // z = M^{-1} r for active columns, CG to relative residual itol (zero start), in the
+  // Chronopoulos-Gear form of cgcg: one sum and one barrier per iteration where the
+  // Hestenes-Stiefel form takes two sums and a barrier.
+  T* const r = (T*)a.r;
+  T* const z = (T*)a.z;
+  T* const ir = (T*)a.ir;
+  T* const ip = (T*)a.ip;
+  T* const iw = (T*)a.iq;
+  T* const is = (T*)a.is;
+  const int m = a.m;
+  const int64_t n = a.n;
+  T acc[MT], acc2[MT];
+  for (int c = threadIdx.x; c < m; c += blockDim.x) {
+    s.iact[c] = s.act[c] && s.rr[c] > 0.0;
+    s.irn0[c] = a.itol * a.itol * s.rr[c];
+    s.iit[c] = 0;
+  }
+  __syncthreads();
+  FOR_BLOCK_SHARE(i, n)
+    _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
+      if (s.act[c]) {
+        z[wix<MT>(i, c)] = T(0);
+        ir[wix<MT>(i, c)] = r[wix<MT>(i, c)];
+      }
+  if (!grid_sync(a.bar)) return false;
+  for (int j = 1;; ++j) {
+    int any = 0;
+    _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) any |= s.iact[c];
+    if (!any) break;
+#pragma unroll
+    for (int c = 0; c < MT; ++c) acc[c] = acc2[c] = T(0);
+    spmv_cols<MT, T, true>(a.M, ir, 0, iw, m, s.iact, ir, acc, acc2);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val, acc2, s.val2)) return false;
+    if (threadIdx.x < m) {
+      const int c = threadIdx.x;
+      if (s.iact[c]) {
+        const double g = s.val2[c], dl = s.val[c];
+        if (j > 1 && g <= s.irn0[c]) {
+          s.iact[c] = 0;  // converged after update j - 1
+        } else if (j <= a.imaxit) {
+          const double be = j > 1 ? g / s.irr[c] : 0.0;
+          const double den = j > 1 ? fma(-be * be, s.iden[c], dl) : dl;  // beta gamma / alpha' = beta^2 den'
+          if (!(den > 0.0)) s.iact[c] = 0;
+          s.irr[c] = g;
+          s.iden[c] = den;
+          s.ia[c] = g / den;
+          s.val2[c] = be;
+          s.iit[c] = j;
+        }
+      }
+    }
+    __syncthreads();
+    if (j > a.imaxit) break;
+    const bool first = (j == 1);
+    FOR_BLOCK_SHARE(i, n)
+      _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
+        if (s.iact[c]) {
+          const int64_t o = wix<MT>(i, c);
+          const T be = (T)s.val2[c], al = (T)s.ia[c];
+          const T r0 = ir[o];
+          const T sn = first ? iw[o] : fma(be, is[o], iw[o]);
+          const T pn = first ? r0 : fma(be, ip[o], r0);
+          ir[o] = fma(-al, sn, r0);
+          is[o] = sn;
+          ip[o] = pn;
+          z[o] = fma(al, pn, z[o]);
+        }
+    if (!grid_sync(a.bar)) return false;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    long long t = 0;
+    _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) t += s.iit[c];
+    *a.in_out += t;
+  }
+  return true;
+}
+
+template <int MT, typename T>
+__device__ __forceinline__ bool inner_solve(const SolverArgs& a, Sh<MT>& s) {
+  if constexpr (sizeof(T) == 8)
+    return inner_cg<MT, T>(a, s);
+  else
+    return inner_cg_hs<MT, T>(a, s);
 }
 
 // ---- mode 3: the V-cycle preconditioner z = V(r), FP32 work
@@ -618,7 +719,7 @@ __device__ __forceinline__ bool cheb_prec(const SolverArgs& a, const int* act) {
   return true;
 }
 
-// Mode 0: CG in the Chronopoulos-Gear form: r^T r and r^T A r are both
+// Modes 0 and 2: CG in the Chronopoulos-Gear form: r^T r and r^T A r are both
 // formed in the SpMV pass (w = A r), so an iteration has one reduction round
 // (block sums, grid barrier, partials) and one plain grid barrier before the
 // next SpMV; same iterates as Hestenes-Stiefel CG in exact arithmetic.  The
@@ -643,9 +744,7 @@ __device__ bool cgcg(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = acc2[c] = T(0);
     spmv_cols<MT, T, true>(a.A, r, 0, w, m, s.act, r, acc, acc2);
-    write_partials<MT, T>(a.red, 0, m, acc, s, acc2, 1);
-    if (!grid_sync(a.bar)) return false;
-    reduce_slot<MT>(a.red, 0, m, s.val, 1, s.val2);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val, acc2, s.val2)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -673,19 +772,32 @@ __device__ bool cgcg(const SolverArgs& a, Sh<MT>& s) {
     if (it > a.maxit) break;  // columns still active report no convergence
     // p = r + beta p, s = w + beta s, x += alpha p, r -= alpha s
     const bool first = (it == 1);
-    FOR_BLOCK_SHARE(i, n)
-      _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
-        if (s.act[c]) {
-          const int64_t o = wix<MT>(i, c), ox = i + c * ld;
-          const T be = (T)s.val2[c], al = (T)s.alpha[c];
-          const T rv0 = r[o];
-          const T pv = first ? rv0 : fma(be, p[o], rv0);
-          const T svv = first ? w[o] : fma(be, sv[o], w[o]);
-          p[o] = pv;
-          sv[o] = svv;
-          x[ox] = fma(al, pv, x[ox]);
-          r[o] = fma(-al, svv, rv0);
-        }
+    auto update = [&](int64_t i, int c, T wv) {
+      const int64_t o = wix<MT>(i, c), ox = i + c * ld;
+      const T be = (T)s.val2[c], al = (T)s.alpha[c];
+      const T rv0 = r[o];
+      const T pv = first ? rv0 : fma(be, p[o], rv0);
+      const T svv = first ? wv : fma(be, sv[o], wv);
+      p[o] = pv;
+      sv[o] = svv;
+      x[ox] = fma(al, pv, x[ox]);
+      r[o] = fma(-al, svv, rv0);
+    };
+    if (a.mode == 2) {  // w projected per segment; r stays in range(P), so delta needs no projection
+      FOR_BLOCK_SHARE(sg, a.nseg) {
+        const int32_t s0 = a.seg_ptr[sg], s1 = a.seg_ptr[sg + 1];
+        _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
+          if (s.act[c]) {
+            T t = T(0);
+            for (int32_t i = s0; i < s1; ++i) t = fma((T)a.phi[i], w[wix<MT>(i, c)], t);
+            for (int32_t i = s0; i < s1; ++i) update(i, c, fma(-(T)a.phi[i], t, w[wix<MT>(i, c)]));
+          }
+      }
+    } else {
+      FOR_BLOCK_SHARE(i, n)
+        _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
+          if (s.act[c]) update(i, c, w[wix<MT>(i, c)]);
+    }
     if (!grid_sync(a.bar)) return false;
   }
   return true;
@@ -756,15 +868,12 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
       _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) a.x64[i + c * ld] = 0.0;
   if (!grid_sync(a.bar)) return false;
   reliable_residual<MT, T>(a, all1, r, dacc);
-  write_partials<MT, double>(a.red, 1, m, dacc, s);
+  double bacc[MT];
 #pragma unroll
-  for (int c = 0; c < MT; ++c) dacc[c] = 0.0;
+  for (int c = 0; c < MT; ++c) bacc[c] = 0.0;
   FOR_BLOCK_SHARE(i, n)
-    _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) dacc[c] = fma(a.b64[i + c * ld], a.b64[i + c * ld], dacc[c]);
-  write_partials<MT, double>(a.red, 0, m, dacc, s);
-  if (!grid_sync(a.bar)) return false;
-  reduce_slot<MT>(a.red, 0, m, s.bn);
-  reduce_slot<MT>(a.red, 1, m, s.rr);
+    _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) bacc[c] = fma(a.b64[i + c * ld], a.b64[i + c * ld], bacc[c]);
+  if (!sum_cols<MT, double>(a.bar, s, m, bacc, s.bn, dacc, s.rr)) return false;
   if (threadIdx.x < m) {
     const int c = threadIdx.x;
     s.bn[c] = sqrt(s.bn[c]);
@@ -788,9 +897,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
     spmv_cols<MT, T, true>(a.A, p, 0, q, m, s.act, p, acc);
-    write_partials<MT, T>(a.red, 0, m, acc, s);
-    if (!grid_sync(a.bar)) return false;
-    reduce_slot<MT>(a.red, 0, m, s.val);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -818,9 +925,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
           r[o] = rv;
           acc[c] = fma(rv, rv, acc[c]);
         }
-    write_partials<MT, T>(a.red, 1, m, acc, s);
-    if (!grid_sync(a.bar)) return false;
-    reduce_slot<MT>(a.red, 1, m, s.val2);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val2)) return false;
     // the recurrence drifts from the true residual: replace it after every
     // two decades of reduction and before accepting convergence
     int need = 0;
@@ -838,9 +943,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
         dacc[c] = 0.0;
       }
       reliable_residual<MT, T>(a, msk, r, dacc);  // x64 complete: barrier above
-      write_partials<MT, double>(a.red, 2, m, dacc, s);
-      if (!grid_sync(a.bar)) return false;
-      reduce_slot<MT>(a.red, 2, m, s.val2);  // true residuals replace the recurrence ones
+      if (!sum_cols<MT, double>(a.bar, s, m, dacc, s.val2)) return false;  // true residuals replace the recurrence ones
       if (threadIdx.x < m) {
         const int c = threadIdx.x;
         if (s.act[c]) {
@@ -1086,9 +1189,7 @@ __device__ bool dd_true_residual(const SolverArgs& a, Sh<MT>& s, const int* mask
       r[o] = dd_of(rv);
       acc[c] = fma(rv, rv, acc[c]);
     }
-  write_partials<MT, double>(a.red, 3, m, acc, s);
-  if (!grid_sync(a.bar)) return false;
-  reduce_slot<MT>(a.red, 3, m, rr);
+  if (!sum_cols<MT, double>(a.bar, s, m, acc, rr)) return false;
   return true;
 }
 
@@ -1107,6 +1208,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) dd_cg_kernel(SolverArgs 
   __shared__ double s_true[MT], s_last[MT];
   __shared__ long long s_base[MT];
   grid_sync_init();
+  comm_init(s.comm);
   const double* __restrict__ b = (const double*)a.b;
   double* __restrict__ x = (double*)a.x;
   dd* const r = (dd*)a.r;
@@ -1135,9 +1237,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) dd_cg_kernel(SolverArgs 
       }
       acc[c] = fma(b[ox], b[ox], acc[c]);
     }
-  write_partials<MT, double>(a.red, 2, m, acc, s);
-  if (!grid_sync(a.bar)) return;
-  reduce_slot<MT>(a.red, 2, m, s.bn);
+  if (!sum_cols<MT, double>(a.bar, s, m, acc, s.bn)) return;
   if (!dd_true_residual<MT>(a, s, all1, !a.x0, s_true)) return;
   if (threadIdx.x < m) {
     const int c = threadIdx.x;
@@ -1263,6 +1363,7 @@ template <int MT, typename T, int VC>
 __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs a) {
   __shared__ Sh<MT> s;
   grid_sync_init();
+  comm_init(s.comm);
   T* const b = (T*)a.b;
   T* const x = (T*)a.x;
   T* const r = (T*)a.r;
@@ -1343,11 +1444,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
         acc2[c] = fma(rv, rv, acc2[c]);
       }
   }
-  write_partials<MT, T>(a.red, 0, m, acc, s);
-  write_partials<MT, T>(a.red, 1, m, acc2, s);
-  if (!grid_sync(a.bar)) return;
-  reduce_slot<MT>(a.red, 0, m, s.bn);
-  reduce_slot<MT>(a.red, 1, m, s.rr);
+  if (!sum_cols<MT, T>(a.bar, s, m, acc, s.bn, acc2, s.rr)) return;
   if (threadIdx.x < m) {
     const int c = threadIdx.x;
     s.bn[c] = sqrt(s.bn[c]);
@@ -1358,7 +1455,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
   FOR_BLOCK_SHARE(i, n)  // zero right-hand sides give x = 0
     _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
       if (s.bn[c] == 0.0) x[i + c * ld] = T(0);
-  if (a.mode == 0) {
+  if (a.mode == 0 || (sizeof(T) == 8 && a.mode == 2)) {  // FP32 keeps mode 2 in the loop below
     if (!cgcg<MT, T>(a, s)) return;
     if (blockIdx.x == 0 && threadIdx.x < m) {
       a.it_out[threadIdx.x] = s.it[threadIdx.x];
@@ -1367,9 +1464,10 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
     return;
   }
   T* zv = r;
-  if (a.mode == 1 || a.mode == 3 || a.mode == 4) {
+  const bool prec = sizeof(T) == 8 || a.mode != 2;  // FP64 comes here with a preconditioner only
+  if (prec) {
     if (a.mode == 1) {
-      if (!inner_cg<MT, T>(a, s)) return;
+      if (!inner_solve<MT, T>(a, s)) return;
     } else if constexpr (sizeof(T) == 8 && VC == 1) {
       if (a.mode == 4) {
         if (!cheb_prec<MT>(a, s.act)) return;
@@ -1383,9 +1481,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
     FOR_BLOCK_SHARE(i, n)
       _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
         if (s.act[c]) acc[c] = fma(r[wix<MT>(i, c)], z[wix<MT>(i, c)], acc[c]);
-    write_partials<MT, T>(a.red, 0, m, acc, s);
-    if (!grid_sync(a.bar)) return;
-    reduce_slot<MT>(a.red, 0, m, s.rz);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.rz)) return;
   } else {
     if (threadIdx.x < m) s.rz[threadIdx.x] = s.rr[threadIdx.x];
     __syncthreads();
@@ -1403,9 +1499,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
     spmv_cols<MT, T, true>(a.A, p, 0, q, m, s.act, p, acc);
-    write_partials<MT, T>(a.red, 0, m, acc, s);
-    if (!grid_sync(a.bar)) return;
-    reduce_slot<MT>(a.red, 0, m, s.val);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -1422,7 +1516,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
     // x += alpha p, r -= alpha q (mode 2: q projected per segment), r^T r
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
-    if (a.mode == 2) {
+    if (!prec) {
       FOR_BLOCK_SHARE(sg, a.nseg) {
         const int32_t s0 = a.seg_ptr[sg], s1 = a.seg_ptr[sg + 1];
         _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) {
@@ -1452,9 +1546,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
             acc[c] = fma(rv, rv, acc[c]);
           }
     }
-    write_partials<MT, T>(a.red, 1, m, acc, s);
-    if (!grid_sync(a.bar)) return;
-    reduce_slot<MT>(a.red, 1, m, s.val2);
+    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val2)) return;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -1463,7 +1555,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
       }
     }
     __syncthreads();
-    if (a.mode == 1 || a.mode == 3 || a.mode == 4) {
+    if (prec) {
       // columns that just converged (-1) need no preconditioning
       if (threadIdx.x < m) {
         const int c = threadIdx.x;
@@ -1472,7 +1564,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
       }
       __syncthreads();
       if (a.mode == 1) {
-        if (!inner_cg<MT, T>(a, s)) return;
+        if (!inner_solve<MT, T>(a, s)) return;
       } else if constexpr (sizeof(T) == 8 && VC == 1) {
         if (a.mode == 4) {
           if (!cheb_prec<MT>(a, s.act)) return;
@@ -1489,11 +1581,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
             acc[c] = fma(r[o], z[o], acc[c]);
             acc2[c] = fma(z[o], q[o], acc2[c]);
           }
-      write_partials<MT, T>(a.red, 0, m, acc, s);
-      write_partials<MT, T>(a.red, 1, m, acc2, s);
-      if (!grid_sync(a.bar)) return;
-      reduce_slot<MT>(a.red, 0, m, s.val);
-      reduce_slot<MT>(a.red, 1, m, s.val2);
+      if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val, acc2, s.val2)) return;
       if (threadIdx.x < m) {
         const int c = threadIdx.x;
         if (s.act[c]) {
