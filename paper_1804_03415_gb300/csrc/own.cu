@@ -281,12 +281,13 @@ __global__ void __launch_bounds__(kOwnThreads, 1) own_cg_kernel(SolverArgs a, Ow
     __syncthreads();
     if (!CL && s.comm.fail) return;  // a cluster's blocks are told with the next sums
     // w = A r; delta = r^T w, gamma = r^T r.  A small share waits for the FMA chains of its widest
-    // rows: a slice's entries are dealt to several warps then, and their sums added afterwards.  Up
-    // to kOwnUnits parts in all, three rounds of the warps; from 13 slices on the chains overlap
-    // anyway.
+    // rows: a slice's entries are dealt to several warps then, and their sums added afterwards (a
+    // barrier and the adds, about 400 cycles, against 85 an entry: parts of eight entries at
+    // least).  Up to kOwnUnits parts in all, three rounds of the warps; from 13 slices on the
+    // chains overlap anyway.
     acc = acc2 = 0.0;
     int parts = 1;
-    while (parts < 8 && nsl * parts * 2 <= kOwnUnits) parts *= 2;
+    while (parts < 8 && nsl * parts * 2 <= kOwnUnits && smeta[0].y >= 16 * parts) parts *= 2;
     auto row_done = [&](int q, double ax) {
       const double r0 = rv[q];
       wv[q] = ax;

@@ -4,10 +4,11 @@
 // Refinement (Algorithm 5: CG on B^(l) = U^T A U and the warm-started PCG).
 //
 // One cooperative launch (one 1024-thread block per SM) runs a whole solve
-// for m <= MT right-hand sides (column-major,
-// leading dimension ld).  Scalars never leave the device: each block writes its partial sums, a bounded grid barrier
-// follows, and every block then reduces the same partials in the same order,
-// so all blocks take identical decisions.
+// for m <= MT right-hand sides (column-major, leading dimension ld).  (FP64 CG
+// on one right-hand side has its own kernel, own.cu, and comes here only where
+// that one does not fit.)  Scalars never leave the device: sums go through
+// tagged words (grid_comm.cuh), every block adding the same ones in the same
+// order, so all blocks take identical decisions.
 //
 // GB300 retires about one FP64 warp-instruction per 16 SM cycles, so the
 // kernel is organised to issue as few FP64 instructions as the arithmetic
