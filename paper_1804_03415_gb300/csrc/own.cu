@@ -20,7 +20,7 @@
 //
 // Measured, cycles per iteration at 2.07 GHz, before -> after (solve_kernel
 // on the same matrices): 64 x 64 grid operator 19.6k -> 9.3k; geometric graph
-// of 50k rows 37k -> 20k; point-cloud graph of 200k rows 100k -> 60k.
+// of 50k rows 37k -> 20k; point-cloud graph of 200k rows 98k -> 55k.
 //
 // Two instances:
 //   grid     a cooperative launch over many SMs, sums and barriers of
