@@ -176,6 +176,8 @@ template <bool CL>
 __global__ void __launch_bounds__(kOwnThreads, 1) own_cg_kernel(SolverArgs a, OwnPlan pl) {
   __shared__ OwnSh s;
   comm_init(s.comm);
+  // a block's shared memory may be written by its peers once it runs: the first sums store into it
+  if constexpr (CL) cluster_barrier();
   constexpr int NT = kOwnThreads, nw = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Sell& A = a.A;

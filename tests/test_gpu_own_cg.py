@@ -80,3 +80,17 @@ def test_own_cg_beyond_shared_memory():
     A = matrix("path", 1_200_000)
     b = np.random.default_rng(6).standard_normal(A.shape[0])
     assert np.linalg.norm(b - A @ solve(A, b)) <= 2 * TOL * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("blocks", range(3, 17))
+def test_own_cg_cluster_sizes(blocks):
+    """Every cluster size from 3 to 16 blocks (a block per SELL slice of 32 rows), the last slice ragged; rows of one
+    entry leave a block nothing to do before the sums that cross the cluster."""
+    for kind in ("rand", "path", "diag"):
+        n = 32 * blocks - 5
+        A = matrix(kind, n)
+        b = np.random.default_rng(blocks).standard_normal(n)
+        x = solve(A, b)
+        nb = np.linalg.norm(b)
+        assert np.linalg.norm(b - A @ x) <= 2 * TOL * nb
+        assert np.linalg.norm(x - spl.spsolve(A.tocsc(), b)) <= 2 * TOL * nb
