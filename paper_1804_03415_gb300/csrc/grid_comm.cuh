@@ -176,7 +176,12 @@ __device__ __forceinline__ bool grid_sums(const GridBarrier& b, CommSh& cs, cons
     } else {
       if (blockIdx.x % gs == 0) {  // first of its group
         ok = poll_sum(b, sl + blockIdx.x, min(gs, G - blockIdx.x), tag, &t);
-        if (FENCE) fence_gpu();
+        if (FENCE) {
+          // the group's sum stands for the writes of every block whose word a lane has read: each
+          // lane's fence is complete before lane 0's store (votes and shuffles order no memory)
+          fence_gpu();
+          __syncwarp();
+        }
         if (ok && lane == 0)
           st_tagged(sl + G + blockIdx.x / gs, (unsigned long long)__double_as_longlong(t), tag);
       }
