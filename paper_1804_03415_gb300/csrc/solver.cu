@@ -28,7 +28,12 @@
 //   1  flexible PCG on A with preconditioner M applied by an inner CG;
 //      beta = z+^T (r+ - r) / (r^T z)  (Golub and Ye, 1999), computed as
 //      -alpha z+^T q / (r^T z) since r+ - r = -alpha q.
-//   2  the same on P A P with P = I - Phi Phi^T applied segment by segment.  Since
+//   2  CG on P A P with P = I - Phi Phi^T applied segment by segment, in the
+//      Hestenes-Stiefel form: two sums and a barrier per iteration.  (In the form
+//      of mode 0 r leaves the range of P by rounding, r^T A r then holds more than
+//      the recurrence takes off, and the step length's denominator loses its sign:
+//      at 1e-13 a 64 x 64 grid operator with a = 10^U(-2,2), 865 iterations here,
+//      ended there as not SPD.)  Since
 //      U of Section 2.3 has orthonormal columns and U U^T = P on each patch,
 //      this is CG on B = U^T A U in the coordinates U g (same iterates); the
 //      solution returned is x = U g.
@@ -720,7 +725,7 @@ __device__ __forceinline__ bool cheb_prec(const SolverArgs& a, const int* act) {
   return true;
 }
 
-// Modes 0 and 2: CG in the Chronopoulos-Gear form: r^T r and r^T A r are both
+// Mode 0: CG in the Chronopoulos-Gear form: r^T r and r^T A r are both
 // formed in the SpMV pass (w = A r), so an iteration has one reduction round
 // (block sums, grid barrier, partials) and one plain grid barrier before the
 // next SpMV; same iterates as Hestenes-Stiefel CG in exact arithmetic.  The
@@ -773,32 +778,19 @@ __device__ bool cgcg(const SolverArgs& a, Sh<MT>& s) {
     if (it > a.maxit) break;  // columns still active report no convergence
     // p = r + beta p, s = w + beta s, x += alpha p, r -= alpha s
     const bool first = (it == 1);
-    auto update = [&](int64_t i, int c, T wv) {
-      const int64_t o = wix<MT>(i, c), ox = i + c * ld;
-      const T be = (T)s.val2[c], al = (T)s.alpha[c];
-      const T rv0 = r[o];
-      const T pv = first ? rv0 : fma(be, p[o], rv0);
-      const T svv = first ? wv : fma(be, sv[o], wv);
-      p[o] = pv;
-      sv[o] = svv;
-      x[ox] = fma(al, pv, x[ox]);
-      r[o] = fma(-al, svv, rv0);
-    };
-    if (a.mode == 2) {  // w projected per segment; r stays in range(P), so delta needs no projection
-      FOR_BLOCK_SHARE(sg, a.nseg) {
-        const int32_t s0 = a.seg_ptr[sg], s1 = a.seg_ptr[sg + 1];
-        _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
-          if (s.act[c]) {
-            T t = T(0);
-            for (int32_t i = s0; i < s1; ++i) t = fma((T)a.phi[i], w[wix<MT>(i, c)], t);
-            for (int32_t i = s0; i < s1; ++i) update(i, c, fma(-(T)a.phi[i], t, w[wix<MT>(i, c)]));
-          }
-      }
-    } else {
-      FOR_BLOCK_SHARE(i, n)
-        _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
-          if (s.act[c]) update(i, c, w[wix<MT>(i, c)]);
-    }
+    FOR_BLOCK_SHARE(i, n)
+      _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
+        if (s.act[c]) {
+          const int64_t o = wix<MT>(i, c), ox = i + c * ld;
+          const T be = (T)s.val2[c], al = (T)s.alpha[c];
+          const T rv0 = r[o];
+          const T pv = first ? rv0 : fma(be, p[o], rv0);
+          const T svv = first ? w[o] : fma(be, sv[o], w[o]);
+          p[o] = pv;
+          sv[o] = svv;
+          x[ox] = fma(al, pv, x[ox]);
+          r[o] = fma(-al, svv, rv0);
+        }
     if (!grid_sync(a.bar)) return false;
   }
   return true;
@@ -1456,7 +1448,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
   FOR_BLOCK_SHARE(i, n)  // zero right-hand sides give x = 0
     _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
       if (s.bn[c] == 0.0) x[i + c * ld] = T(0);
-  if (a.mode == 0 || (sizeof(T) == 8 && a.mode == 2)) {  // FP32 keeps mode 2 in the loop below
+  if (a.mode == 0) {
     if (!cgcg<MT, T>(a, s)) return;
     if (blockIdx.x == 0 && threadIdx.x < m) {
       a.it_out[threadIdx.x] = s.it[threadIdx.x];
@@ -1465,7 +1457,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
     return;
   }
   T* zv = r;
-  const bool prec = sizeof(T) == 8 || a.mode != 2;  // FP64 comes here with a preconditioner only
+  const bool prec = a.mode != 2;
   if (prec) {
     if (a.mode == 1) {
       if (!inner_solve<MT, T>(a, s)) return;

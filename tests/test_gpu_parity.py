@@ -525,3 +525,25 @@ def test_wide_solve_replays_its_cuda_graph():
     err = np.abs(lam - lam64)
     assert np.all(err <= np.maximum(1e-9 * np.abs(lam64), 1e-9 * st64["norm_A"])), float((err / lam64).max())
     h.close()
+
+
+@pytest.mark.parametrize("size", [24, 40, 48, 64])
+def test_level_bsolve_deep(size):
+    """The complement solve of badly conditioned operators (a = 10^U(-2,2)) down to 1e-13: the residual that the
+    recurrence carries meets the tolerance, and the true one differs from it by the rounding of its updates, at most
+    (row length + 4) eps ||A|| ||x|| an iteration."""
+    tol = 1e-13
+    A = W.fd2d(size, seed=3)
+    D = OM.build(A, OM.BuildOpts(n_coarse=20))
+    lev, S = D.levels[0], D.A(0)
+    h = _handle(A, n_coarse=20)
+    for seed in (3, 4, 5):
+        q = np.random.default_rng(seed).standard_normal(A.n)
+        x = torch.zeros(A.n, dtype=torch.float64, device="cuda")
+        its = h.level_bsolve(1, _dev(q), x, tol)
+        xh = x.cpu().numpy()
+        b = OM.Ut_apply(lev, q)
+        res = np.linalg.norm(b - OM.Ut_apply(lev, S @ xh))
+        rounding = 9 * its * np.finfo(float).eps * abs(S).sum(1).max() * np.linalg.norm(xh)
+        assert res <= tol * np.linalg.norm(b) + rounding
+    h.close()
