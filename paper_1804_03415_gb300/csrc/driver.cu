@@ -59,6 +59,10 @@ struct OwnShares {
   const uint16_t* lcol = nullptr;
 };
 
+// partial sums of one launch on at most 512 blocks: [4][4][grid] of the double-float
+// CG, then [2][8][grid]
+constexpr size_t kRedDoubles = size_t(2) * 16 * 512;
+
 struct Workspace {
   std::map<std::pair<int, int>, OwnShares> shares;  // by (level, grid)
   int cluster16 = -1;  // a cluster of 16 blocks can run here (-1: not asked yet)
@@ -151,7 +155,7 @@ Workspace* get_ws(mmd_handle* h) {
   CK(cudaMemset(ws->bar, 0, 64 * sizeof(unsigned)));
   CK(cudaMalloc(&ws->status, sizeof(int)));
   CK(cudaMemset(ws->status, 0, sizeof(int)));
-  CK(cudaMalloc(&ws->red, sizeof(double) * 4 * 8 * 512));
+  CK(cudaMalloc(&ws->red, sizeof(double) * kRedDoubles));
   CK(cudaMalloc(&ws->it_out, sizeof(int64_t) * 8));
   CK(cudaMalloc(&ws->in_out, sizeof(int64_t)));
   CK(cudaMalloc(&ws->conv, sizeof(int) * 8));
@@ -657,7 +661,8 @@ struct Ctx {
       a.itol = 0.1 * tol;
       a.maxit = maxit;
       a.imaxit = std::min(maxit, 1000);
-      a.red = buf<double>(ws, "red" + ls, size_t(4) * 8 * 512);
+      a.red = buf<double>(ws, "red" + ls, kRedDoubles);
+      a.sums = a.red + kRedDoubles / 2;
       a.it_out = it_all + c0;
       a.in_out = inn_all + l;
       a.conv = cv_all + c0;
@@ -669,7 +674,7 @@ struct Ctx {
       if (mode == 3) set_mg(a, mg_deg, mg_only, l);
       if (mode == 4) set_poly(a, poly_deg, l);
       CK(cudaMemsetAsync(bar, 0, sizeof(unsigned) * 64, sl));
-      comm_words(a.bar, ls, MT, grid, sl);
+      if (grid <= kTaggedBlocks) comm_words(a.bar, ls, MT, grid, sl);
       CK(launch_solver(a, MT, grid, sl));
       after_launch();
     }
@@ -804,7 +809,7 @@ struct Ctx {
     bool cl = false;
     if (MT != 1 || a.mode != 0 || a.fp32 || a.df || a.b64 ||
         !own_choice(k, coop_grid_cap() > 0 ? coop_grid_cap() : ws->nsm, &plan, &g, &cl)) {
-      comm_words(a.bar, "", MT, grid, st);
+      if (grid <= kTaggedBlocks) comm_words(a.bar, "", MT, grid, st);
       return launch_solver(a, MT, grid, st);
     }
     if (!cl) comm_words(a.bar, "", MT, g, st);
@@ -894,6 +899,7 @@ struct Ctx {
       a.maxit = maxit;
       a.imaxit = std::min(maxit, 1000);
       a.red = ws->red;
+      a.sums = a.red + kRedDoubles / 2;
       a.it_out = ws->it_out;
       a.in_out = ws->in_out;
       a.conv = ws->conv;

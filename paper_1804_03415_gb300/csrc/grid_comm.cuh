@@ -147,10 +147,14 @@ __host__ __device__ inline unsigned sum_group(unsigned G) {
 // 16-byte words of the tagged sums of nvmax values on G blocks
 __host__ __device__ inline size_t sum_words(int nvmax, unsigned G) { return size_t(2) * nvmax * (G + 32); }
 
+// Largest grid whose fenced sums go through tagged words.
+constexpr int kTaggedBlocks = 16;
+
 // Grid-wide sums dst[v] (shared) of nv values in every block, all blocks
 // adding the same partials in the same order.  FENCE: also a full barrier
-// (what any thread wrote before it is seen after it); without, only the sums
-// are exchanged, and a block has read everything it reads before it.
+// (what any thread wrote before it is seen after it), on at most
+// kTaggedBlocks blocks, each of which reads every other's word; without, only
+// the sums are exchanged, and a block has read everything it reads before it.
 // b.slots: sum_words(nvmax, G) zeroed words; a block overwrites the words of
 // sum R with those of sum R + 2, after every block has published sum R + 1
 // and so has read sum R.  blockDim >= 32 nv.
@@ -159,7 +163,7 @@ __device__ __forceinline__ bool grid_sums(const GridBarrier& b, CommSh& cs, cons
                                           int nvmax, int lim, double* quart, double* dst) {
   const int wpc = block_sums(part, stride, nv, lim, quart);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned G = gridDim.x, gs = sum_group(G);
+  const unsigned G = gridDim.x, gs = FENCE ? 1 : sum_group(G);
   const unsigned tag = cs.nred + 1;
   if (w < nv) {
     ulonglong2* sl = b.slots + (size_t(tag & 1u) * nvmax + w) * (G + 32);
@@ -176,12 +180,6 @@ __device__ __forceinline__ bool grid_sums(const GridBarrier& b, CommSh& cs, cons
     } else {
       if (blockIdx.x % gs == 0) {  // first of its group
         ok = poll_sum(b, sl + blockIdx.x, min(gs, G - blockIdx.x), tag, &t);
-        if (FENCE) {
-          // the group's sum stands for the writes of every block whose word a lane has read: each
-          // lane's fence is complete before lane 0's store (votes and shuffles order no memory)
-          fence_gpu();
-          __syncwarp();
-        }
         if (ok && lane == 0)
           st_tagged(sl + G + blockIdx.x / gs, (unsigned long long)__double_as_longlong(t), tag);
       }

@@ -87,7 +87,8 @@ struct SolverArgs {
   double* x64;
   double tol, itol;
   int maxit, imaxit;
-  double* red;         // [4][MT][grid]
+  double* red;         // [4][MT][grid] (df)
+  double* sums;        // [2][2 MT][grid] partial sums of the blocks
   int64_t* it_out;     // [m]
   int64_t* in_out;     // [1], accumulated
   int* conv;           // [m]

@@ -6,9 +6,8 @@
 // One cooperative launch (one 1024-thread block per SM) runs a whole solve
 // for m <= MT right-hand sides (column-major, leading dimension ld).  (FP64 CG
 // on one right-hand side has its own kernel, own.cu, and comes here only where
-// that one does not fit.)  Scalars never leave the device: sums go through
-// tagged words (grid_comm.cuh), every block adding the same ones in the same
-// order, so all blocks take identical decisions.
+// that one does not fit.)  Scalars never leave the device: every block adds the
+// blocks' partial sums in the same order, so all blocks take identical decisions.
 //
 // GB300 retires about one FP64 warp-instruction per 16 SM cycles, so the
 // kernel is organised to issue as few FP64 instructions as the arithmetic
@@ -90,9 +89,15 @@ __device__ __forceinline__ int64_t share_hi(int64_t n) { return n * (blockIdx.x 
 extern __shared__ double g_part[];
 
 // Grid-wide sums of the threads' acc[c] into dst[c], c < m, and of acc2[c]
-// into dst2[c] (both shared), and a full barrier: grid_comm.cuh.
+// into dst2[c] (both shared), and a full barrier: tagged words (grid_comm.cuh)
+// on at most kTaggedBlocks blocks, else every block's partials, the arrival
+// counter's barrier, and warp v of every block adds the partials of value v.
+// Tagged words save a round trip, but on many blocks their polls and stores
+// keep each other waiting.  Tagged -> counter: level-1 operator of a 5,000-row
+// graph (few blocks) 28.3 -> 30.4 ms, of a 100k-row graph (96 blocks) 56.8 ->
+// 53.4 ms; four columns on a 160 x 160 operator (152 blocks) 89.0 -> 84.0 ms.
 template <int MT, typename T>
-__device__ __forceinline__ bool sum_cols(const GridBarrier& bar, Sh<MT>& s, int m, const T* acc, double* dst,
+__device__ __forceinline__ bool sum_cols(const SolverArgs& a, Sh<MT>& s, int m, const T* acc, double* dst,
                                          const T* acc2 = nullptr, double* dst2 = nullptr) {
   constexpr int NT = threads_for<MT>();
   const int tid = threadIdx.x, nv = acc2 ? 2 * m : m;
@@ -102,8 +107,28 @@ __device__ __forceinline__ bool sum_cols(const GridBarrier& bar, Sh<MT>& s, int 
       g_part[c * NT + tid] = (double)acc[c];
       if (acc2) g_part[(m + c) * NT + tid] = (double)acc2[c];
     }
-  if (!grid_sums<true>(bar, s.comm, g_part, NT, nv, 2 * MT, NT, s.quart, s.sum)) return false;
-  if (tid < nv) (tid < m ? dst : dst2)[tid < m ? tid : tid - m] = s.sum[tid];
+  if (gridDim.x <= kTaggedBlocks) {
+    if (!grid_sums<true>(a.bar, s.comm, g_part, NT, nv, 2 * MT, NT, s.quart, s.sum)) return false;
+    if (tid < nv) (tid < m ? dst : dst2)[tid < m ? tid : tid - m] = s.sum[tid];
+  } else {
+    const int wpc = block_sums(g_part, NT, nv, NT, s.quart);
+    const int G = gridDim.x, w = tid >> 5, lane = tid & 31;
+    // two sets in turn: a block that is one sum ahead leaves the partials that others still read
+    double* const part = a.sums + size_t(s.comm.nred & 1u) * (2 * MT) * G;
+    if (tid < nv) {
+      double t = s.quart[tid * 4];
+      for (int q = 1; q < wpc; ++q) t += s.quart[tid * 4 + q];
+      part[tid * G + blockIdx.x] = t;
+    }
+    if (!grid_sync(a.bar)) return false;
+    if (w < nv) {
+      double t = 0.0;
+      for (int i = lane; i < G; i += 32) t += part[w * G + i];
+      t = warp_sum(t);
+      if (lane == 0) (w < m ? dst : dst2)[w < m ? w : w - m] = t;
+    }
+    if (tid == 0) ++s.comm.nred;  // read again behind the barriers of the next sum
+  }
   __syncthreads();
   return true;
 }
@@ -304,7 +329,7 @@ __device__ bool inner_cg_hs(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
     spmv_cols<MT, T, true>(a.M, ip, 0, iq, m, s.iact, ip, acc);
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return false;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val)) return false;
     if (threadIdx.x < m) s.ia[threadIdx.x] = s.iact[threadIdx.x] ? s.irr[threadIdx.x] / s.val[threadIdx.x] : 0.0;
     __syncthreads();
 #pragma unroll
@@ -319,7 +344,7 @@ __device__ bool inner_cg_hs(const SolverArgs& a, Sh<MT>& s) {
           ir[o] = rv;
           acc[c] = fma(rv, rv, acc[c]);
         }
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return false;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.iact[c]) {
@@ -381,7 +406,7 @@ __device__ bool inner_cg(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = acc2[c] = T(0);
     spmv_cols<MT, T, true>(a.M, ir, 0, iw, m, s.iact, ir, acc, acc2);
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val, acc2, s.val2)) return false;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val, acc2, s.val2)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.iact[c]) {
@@ -750,7 +775,7 @@ __device__ bool cgcg(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = acc2[c] = T(0);
     spmv_cols<MT, T, true>(a.A, r, 0, w, m, s.act, r, acc, acc2);
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val, acc2, s.val2)) return false;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val, acc2, s.val2)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -866,7 +891,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
   for (int c = 0; c < MT; ++c) bacc[c] = 0.0;
   FOR_BLOCK_SHARE(i, n)
     _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m) bacc[c] = fma(a.b64[i + c * ld], a.b64[i + c * ld], bacc[c]);
-  if (!sum_cols<MT, double>(a.bar, s, m, bacc, s.bn, dacc, s.rr)) return false;
+  if (!sum_cols<MT, double>(a, s, m, bacc, s.bn, dacc, s.rr)) return false;
   if (threadIdx.x < m) {
     const int c = threadIdx.x;
     s.bn[c] = sqrt(s.bn[c]);
@@ -890,7 +915,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
     spmv_cols<MT, T, true>(a.A, p, 0, q, m, s.act, p, acc);
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return false;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val)) return false;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -918,7 +943,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
           r[o] = rv;
           acc[c] = fma(rv, rv, acc[c]);
         }
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val2)) return false;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val2)) return false;
     // the recurrence drifts from the true residual: replace it after every
     // two decades of reduction and before accepting convergence
     int need = 0;
@@ -936,7 +961,7 @@ __device__ bool cg_rel(const SolverArgs& a, Sh<MT>& s) {
         dacc[c] = 0.0;
       }
       reliable_residual<MT, T>(a, msk, r, dacc);  // x64 complete: barrier above
-      if (!sum_cols<MT, double>(a.bar, s, m, dacc, s.val2)) return false;  // true residuals replace the recurrence ones
+      if (!sum_cols<MT, double>(a, s, m, dacc, s.val2)) return false;  // true residuals replace the recurrence ones
       if (threadIdx.x < m) {
         const int c = threadIdx.x;
         if (s.act[c]) {
@@ -1182,7 +1207,7 @@ __device__ bool dd_true_residual(const SolverArgs& a, Sh<MT>& s, const int* mask
       r[o] = dd_of(rv);
       acc[c] = fma(rv, rv, acc[c]);
     }
-  if (!sum_cols<MT, double>(a.bar, s, m, acc, rr)) return false;
+  if (!sum_cols<MT, double>(a, s, m, acc, rr)) return false;
   return true;
 }
 
@@ -1230,7 +1255,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) dd_cg_kernel(SolverArgs 
       }
       acc[c] = fma(b[ox], b[ox], acc[c]);
     }
-  if (!sum_cols<MT, double>(a.bar, s, m, acc, s.bn)) return;
+  if (!sum_cols<MT, double>(a, s, m, acc, s.bn)) return;
   if (!dd_true_residual<MT>(a, s, all1, !a.x0, s_true)) return;
   if (threadIdx.x < m) {
     const int c = threadIdx.x;
@@ -1437,7 +1462,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
         acc2[c] = fma(rv, rv, acc2[c]);
       }
   }
-  if (!sum_cols<MT, T>(a.bar, s, m, acc, s.bn, acc2, s.rr)) return;
+  if (!sum_cols<MT, T>(a, s, m, acc, s.bn, acc2, s.rr)) return;
   if (threadIdx.x < m) {
     const int c = threadIdx.x;
     s.bn[c] = sqrt(s.bn[c]);
@@ -1474,7 +1499,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
     FOR_BLOCK_SHARE(i, n)
       _Pragma("unroll") for (int c = 0; c < MT; ++c) if (c < m)
         if (s.act[c]) acc[c] = fma(r[wix<MT>(i, c)], z[wix<MT>(i, c)], acc[c]);
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.rz)) return;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.rz)) return;
   } else {
     if (threadIdx.x < m) s.rz[threadIdx.x] = s.rr[threadIdx.x];
     __syncthreads();
@@ -1492,7 +1517,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
 #pragma unroll
     for (int c = 0; c < MT; ++c) acc[c] = T(0);
     spmv_cols<MT, T, true>(a.A, p, 0, q, m, s.act, p, acc);
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val)) return;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val)) return;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -1539,7 +1564,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
             acc[c] = fma(rv, rv, acc[c]);
           }
     }
-    if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val2)) return;
+    if (!sum_cols<MT, T>(a, s, m, acc, s.val2)) return;
     if (threadIdx.x < m) {
       const int c = threadIdx.x;
       if (s.act[c]) {
@@ -1574,7 +1599,7 @@ __global__ void __launch_bounds__(threads_for<MT>(), 1) solve_kernel(SolverArgs 
             acc[c] = fma(r[o], z[o], acc[c]);
             acc2[c] = fma(z[o], q[o], acc2[c]);
           }
-      if (!sum_cols<MT, T>(a.bar, s, m, acc, s.val, acc2, s.val2)) return;
+      if (!sum_cols<MT, T>(a, s, m, acc, s.val, acc2, s.val2)) return;
       if (threadIdx.x < m) {
         const int c = threadIdx.x;
         if (s.act[c]) {

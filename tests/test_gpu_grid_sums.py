@@ -1,4 +1,4 @@
-"""The fenced grid-wide sum of the persistent solver over grids of one and of two levels, with full and ragged groups.
+"""The fenced grid-wide sum of the persistent solver over small grids (tagged words) and large ones (arrival counter).
 
 A block of three columns on a handle without levels runs one tile on ceil(n / 1024) blocks, at least 16.  Matrices are
 Laplacians + I (||A^{-1}|| <= 1), as in the one-column tests: the true residual is held to twice the tolerance.  The sum
