@@ -767,15 +767,16 @@ struct Ctx {
   }
 
   // One right-hand side of FP64 CG on A^(k) on at most `cap` SMs: the launch
-  // of own.cu; false where it does not fit (a block's rows, their neighbours
-  // and five vectors in one SM's shared memory; about 800k rows) and
-  // solve_kernel runs the solve.  One cluster of 16 SMs while the work (FP64
-  // warp instructions of an iteration: a slice's width and six more) is small,
-  // since its sums take 3,500 cycles against 5,000 and more over a grid (64 x
-  // 64 operator, 1.4k instructions: 4.5 us per iteration against 5.1 on 32
-  // blocks; point-cloud graph of 6,000 rows, 7.7k: 11.1 us against 10.2 on
-  // 76); else a block per two slices, up to every SM (graph of 20,000 rows,
-  // 625 slices: 10.9 us on 152 blocks, 11.9 us on 76).
+  // of own.cu; false where it does not fit or would stage too little of the
+  // matrix (own_plan: 10-nearest-neighbour graphs from about 300k rows, grid
+  // operators from about 400k) and solve_kernel runs the solve.  One cluster of 16 SMs
+  // while the work (FP64 warp instructions of an iteration: a slice's width and
+  // six more) is small, since its sums take 3,500 cycles against 5,000 and more
+  // over a grid; else a block per two slices, up to every SM.  us an iteration,
+  // cluster / grid: 10-nearest-neighbour graphs 2.3k instructions 5.9 / 6.4,
+  // 2.9k 6.3 / 6.4, 3.5k 6.6 / 6.5, 4.1k 6.7 / 6.7, 4.6k 7.1 / 6.7; geometric
+  // graphs 2.8k 6.3 / 7.3, 3.8k 6.6 / 7.0; grid operators 1.4k 4.7 / 5.3, 2.2k
+  // 5.2 / 5.5, 3.2k 6.0 / 5.7; random graphs 1.4k 7.6 / 8.4, 2.4k 9.1 / 9.3.
   bool own_choice(int k, int cap, OwnPlan* plan, int* grid, bool* cluster) {
     const DCSR& A = h->dl[k].A;
     if (plain_cg) return false;

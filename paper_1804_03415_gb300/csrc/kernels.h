@@ -134,6 +134,18 @@ cudaError_t launch_wide_cg(const WideArgs& a, int grid, cudaStream_t st);
 // how one launch lays out its shared memory, and what its blocks read.
 constexpr int kOwnSmem = 224 * 1024;  // dynamic shared memory a block may ask for
 constexpr int kNearMax = 12288;       // rows a block may list
+// Shared memory that the vectors and the listed rows of the largest share have
+// to leave for its matrix entries, unless all of them are staged.  Eight warps
+// stream the rest from L2 more slowly than solve_kernel's 32.  us an iteration,
+// solve_kernel / own_cg_kernel, and the KB left: 10-nearest-neighbour graph on a
+// torus of 200k rows 18.3 / 15.5 (122), 300k 20.9 / 21.0 (83), 400k 24.4 / 27.3
+// (43); 600 x 600 operator 19.3 / 16.6 (67), 700 x 700 22.9 / 23.3 (17); random
+// graph of 4 entries a row, 230k rows 17.7 / 18.4 (55), 300k 18.5 / 24.2 (9).
+// Where hardly any listed row serves two entries, the fetch of the rows is as
+// long as the gathers it replaces, and three quarters have to be staged: random
+// graphs of 8 entries a row, 130k rows (all) 18.3 / 17.4, 150k (69%) 18.2 /
+// 19.1; of 12, 100k (88%) 20.4 / 18.6, 120k (56%) 20.6 / 21.2.
+constexpr int kOwnStaged = 64 * 1024;
 struct OwnPlan {
   int slots = 0;                   // 32 x SELL slices of the largest block share
   int near = 0;                    // room for the listed rows' values
@@ -150,7 +162,8 @@ struct OwnPlan {
 // Shares of equal work: block b takes the slices [first[b], first[b + 1]).
 // sptr: host copy of the slice offsets.
 std::vector<int32_t> own_shares(const int32_t* sptr, int64_t nslices, int grid);
-// near: rows listed by the largest block.  False where the launch does not fit.
+// near: rows listed by the largest block.  False where the launch does not fit
+// or too little of the matrix would be staged.
 bool own_plan(const int32_t* sptr, const int32_t* first, int grid, int near, OwnPlan* out);
 bool near_fits(int64_t n);
 cudaError_t launch_near(const Sell& A, int64_t n, int grid, const int32_t* first, int stride, int32_t* count,

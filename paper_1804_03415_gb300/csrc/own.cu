@@ -476,6 +476,8 @@ bool own_plan(const int32_t* sptr, const int32_t* first, int grid, int near, Own
   if (used > kOwnSmem) return false;
   p.slots = (int)slices * 32;
   p.ents = (int)(std::min<int64_t>((kOwnSmem - used) / 10, ents) & ~int64_t(31));  // slices hold multiples of 32
+  if (p.ents < ents && 10 * p.ents < kOwnStaged) return false;
+  if (4 * int64_t(near) > 3 * ents && 4 * int64_t(p.ents) < 3 * ents) return false;
   p.smem = (int)(used + int64_t(10) * p.ents);
   *out = p;
   return true;
