@@ -455,7 +455,7 @@ std::vector<int32_t> own_shares(const int32_t* sptr, int64_t nslices, int grid) 
   int64_t sl = 0;
   for (int b = 0; b < grid; ++b) {
     const double goal = total * b / grid;
-    while (sl < nslices && (sptr[sl] + sptr[sl + 1]) / 64.0 + 6.0 * sl + 3.0 < goal) ++sl;  // nearest boundary
+    while (sl < nslices && (int64_t(sptr[sl]) + sptr[sl + 1]) / 64.0 + 6.0 * sl + 3.0 < goal) ++sl;  // nearest boundary
     first[b] = (int32_t)sl;
   }
   first[0] = 0;

@@ -43,6 +43,9 @@ int main() {
   CHECK(!plan(12500, 13, 4600, &p));
   CHECK(!plan(6250, 5, 11200, &p));
   CHECK(!plan(4688, 10, 8572, &p) && plan(3125, 13, 8477, &p));
+  // shares stay even up to the largest offsets that 32 bits hold
+  const std::vector<int32_t> wide = offsets(60, 1100000), first = mmd::own_shares(wide.data(), 60, 16);
+  for (int b = 0; b < 16; ++b) CHECK(first[b + 1] - first[b] >= 3 && first[b + 1] - first[b] <= 5);
   std::puts("plans hold");
   return 0;
 }
