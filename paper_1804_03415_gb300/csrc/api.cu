@@ -43,7 +43,8 @@ static int dput(T** p, const std::vector<T>& v) {
 }
 
 // Permute a square CSR symmetrically: new row i' = old perm[i'], columns by iperm.
-static HCSR permute_sym(const HCSR& A, const std::vector<int32_t>& perm, const std::vector<int32_t>& iperm) {
+static HCSR permute_sym(const HCSR& A, const std::vector<int32_t>& perm, const std::vector<int32_t>& iperm,
+                        int threads) {
   HCSR B;
   B.nrows = A.nrows;
   B.ncols = A.ncols;
@@ -51,7 +52,7 @@ static HCSR permute_sym(const HCSR& A, const std::vector<int32_t>& perm, const s
   for (int64_t i = 0; i < A.nrows; ++i) B.rowptr[i + 1] = B.rowptr[i] + (A.rowptr[perm[i] + 1] - A.rowptr[perm[i]]);
   B.col.resize(A.col.size());
   B.val.resize(A.val.size());
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) num_threads(threads)
   for (int64_t i = 0; i < A.nrows; ++i) {
     const int32_t r = perm[i];
     std::vector<std::pair<int32_t, double>> row;
@@ -67,7 +68,8 @@ static HCSR permute_sym(const HCSR& A, const std::vector<int32_t>& perm, const s
 }
 
 // Rows permuted by prow (new i' = old prow[i']), columns renumbered by icol.
-static HCSR permute_rect(const HCSR& A, const std::vector<int32_t>& prow, const std::vector<int32_t>& icol) {
+static HCSR permute_rect(const HCSR& A, const std::vector<int32_t>& prow, const std::vector<int32_t>& icol,
+                         int threads) {
   HCSR B;
   B.nrows = A.nrows;
   B.ncols = A.ncols;
@@ -75,7 +77,7 @@ static HCSR permute_rect(const HCSR& A, const std::vector<int32_t>& prow, const 
   for (int64_t i = 0; i < A.nrows; ++i) B.rowptr[i + 1] = B.rowptr[i] + (A.rowptr[prow[i] + 1] - A.rowptr[prow[i]]);
   B.col.resize(A.col.size());
   B.val.resize(A.val.size());
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) num_threads(threads)
   for (int64_t i = 0; i < A.nrows; ++i) {
     const int32_t r = prow[i];
     std::vector<std::pair<int32_t, double>> row;
@@ -123,7 +125,7 @@ static int autotune_spmv(DCSR& D) {
   return MMD_OK;
 }
 
-static int upload_csr(const HCSR& A, DCSR& D) {
+static int upload_csr(const HCSR& A, DCSR& D, int threads) {
   D.nrows = A.nrows;
   D.ncols = A.ncols;
   D.nnz = A.nnz();
@@ -134,7 +136,7 @@ static int upload_csr(const HCSR& A, DCSR& D) {
   std::vector<float> v32(A.val.begin(), A.val.end());
   if ((rc = dput(&D.val32, v32))) return rc;
   std::vector<float> v2(2 * A.val.size());
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) num_threads(threads)
   for (size_t i = 0; i < A.val.size(); ++i) {
     v2[2 * i] = v32[i];
     v2[2 * i + 1] = (float)(A.val[i] - (double)v32[i]);
@@ -150,7 +152,7 @@ static int upload_csr(const HCSR& A, DCSR& D) {
   std::vector<int32_t> order(n);
   for (int64_t i = 0; i < n; ++i) order[i] = (int32_t)i;
   constexpr int64_t kSigma = 1024;  // torus kNN 200k: 1.2% padding (256: 4.2%, 32: 29%)
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) num_threads(threads)
   for (int64_t w0 = 0; w0 < n; w0 += kSigma) {
     const int64_t w1 = std::min<int64_t>(n, w0 + kSigma);
     std::stable_sort(order.begin() + w0, order.begin() + w1, [&](int32_t a, int32_t b) {
@@ -177,7 +179,7 @@ static int upload_csr(const HCSR& A, DCSR& D) {
   const int64_t tot = sptr[ns];
   std::vector<int32_t> scol(tot);
   std::vector<double> sval(tot, 0.0);
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) num_threads(threads)
   for (int64_t s = 0; s < ns; ++s)
     for (int l = 0; l < 32; ++l) {
       const int32_t r = srow[s * 32 + l];
@@ -204,7 +206,7 @@ static int upload_csr(const HCSR& A, DCSR& D) {
   std::vector<float> sv32(sval.begin(), sval.end());
   if ((rc = dput(&D.s_val32, sv32))) return rc;
   std::vector<float> sv2(2 * tot);
-#pragma omp parallel for schedule(static)
+#pragma omp parallel for schedule(static) num_threads(threads)
   for (int64_t i = 0; i < tot; ++i) {
     const float hi = (float)sval[i];
     sv2[2 * i] = hi;
@@ -304,7 +306,7 @@ static void free_csr(DCSR& D) {
 }
 
 int upload_levels(mmd_handle* h) {
-  const int K = (int)h->levels.size();
+  const int K = (int)h->levels.size(), nt = nthreads_of(&h->bopts);
   h->dl.assign(K + 1, DLevel());
   // device order of level k: patches of level k+1 (natural patch ids, or patch_order[k]), rows ascending inside
   std::vector<std::vector<int32_t>> perm(K + 1), iperm(K + 1), patch_order(K + 1);
@@ -321,8 +323,8 @@ int upload_levels(mmd_handle* h) {
     // scattered rows: compact pieces, patch by patch (a patch where its first
     // row comes); the coarsest of several levels is solved dense and stays
     const HCSR& A = (k == 0) ? h->A0 : h->levels[k - 1].A;
-    if ((k < K || K == 0) && scattered(A, iperm[k])) {
-      const std::vector<int32_t> order = bisection_order(A);
+    if ((k < K || K == 0) && scattered(A, iperm[k], nt)) {
+      const std::vector<int32_t> order = bisection_order(A, nt);
       if (k < K) {
         const HLevel& N = h->levels[k];
         std::vector<uint8_t> done(N.n, 0);
@@ -345,11 +347,11 @@ int upload_levels(mmd_handle* h) {
     DLevel& L = h->dl[k];
     const HCSR& A = (k == 0) ? h->A0 : h->levels[k - 1].A;
     L.n = A.nrows;
-    if ((rc = upload_csr(permute_sym(A, perm[k], iperm[k]), L.A))) return rc;
+    if ((rc = upload_csr(permute_sym(A, perm[k], iperm[k], nt), L.A, nt))) return rc;
     if (k >= 1) {
       const HLevel& H = h->levels[k - 1];
-      if ((rc = upload_csr(permute_sym(H.M, perm[k], iperm[k]), L.M))) return rc;
-      if ((rc = upload_csr(permute_rect(H.psi, perm[k - 1], iperm[k]), L.psi))) return rc;
+      if ((rc = upload_csr(permute_sym(H.M, perm[k], iperm[k], nt), L.M, nt))) return rc;
+      if ((rc = upload_csr(permute_rect(H.psi, perm[k - 1], iperm[k], nt), L.psi, nt))) return rc;
       L.eps = H.eps;
       L.delta = H.delta;
     }
@@ -407,7 +409,7 @@ int upload_levels(mmd_handle* h) {
       for (int k = 0; k < K; ++k) {
         if ((rc = diag_data(k))) return rc;
         const HLevel& H = h->levels[k];
-        if ((rc = upload_csr(transpose(permute_rect(H.psi, perm[k], iperm[k + 1])), h->dl[k + 1].psiT))) return rc;
+        if ((rc = upload_csr(transpose(permute_rect(H.psi, perm[k], iperm[k + 1], nt)), h->dl[k + 1].psiT, nt))) return rc;
       }
       std::vector<float> kinv(inv.begin(), inv.end());  // natural order = device order on level K
       if ((rc = dput(&h->dl[K].kinv32, kinv))) return rc;

@@ -33,6 +33,16 @@
 #include "mmd_internal.h"
 
 namespace mmd {
+
+int nthreads_of(const mmd_build_opts* o) {
+#ifdef _OPENMP
+  return o->threads > 0 ? o->threads : omp_get_max_threads();
+#else
+  (void)o;
+  return 1;
+#endif
+}
+
 namespace {
 
 // ------------------------------------------------------------ small dense
@@ -140,15 +150,6 @@ double entry(const HCSR& A, int r, int c) {
   const int32_t* e = A.col.data() + A.rowptr[r + 1];
   const int32_t* p = std::lower_bound(b, e, c);
   return (p != e && *p == c) ? A.val[p - A.col.data()] : 0.0;
-}
-
-int nthreads_of(const mmd_build_opts* o) {
-#ifdef _OPENMP
-  return o->threads > 0 ? o->threads : omp_get_max_threads();
-#else
-  (void)o;
-  return 1;
-#endif
 }
 
 // ------------------------------------------------------------ 1. partition

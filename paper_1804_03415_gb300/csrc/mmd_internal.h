@@ -108,6 +108,7 @@ namespace mmd {
 
 void set_error(const std::string& msg);
 int build_host(const mmd_csr* A, const mmd_build_opts* o, mmd_handle* h);
+int nthreads_of(const mmd_build_opts* o);  // host threads that the options allow
 int upload_levels(mmd_handle* h);
 void free_device(mmd_handle* h);
 

@@ -12,10 +12,10 @@ namespace mmd {
 // thin rim.  True where more than a quarter of A's entries (in the order
 // given by iperm) lie further than n / 32 from the diagonal: point clouds and
 // geometric graphs numbered at random, not the grid operators.
-bool scattered(const HCSR& A, const std::vector<int32_t>& iperm) {
+bool scattered(const HCSR& A, const std::vector<int32_t>& iperm, int threads) {
   const int64_t far = std::max<int64_t>(512, A.nrows / 32);
   int64_t out = 0;
-#pragma omp parallel for schedule(static) reduction(+ : out)
+#pragma omp parallel for schedule(static) num_threads(threads) reduction(+ : out)
   for (int64_t r = 0; r < A.nrows; ++r)
     for (int32_t e = A.rowptr[r]; e < A.rowptr[r + 1]; ++e)
       out += std::abs(int64_t(iperm[r]) - iperm[A.col[e]]) > far;
@@ -30,7 +30,7 @@ bool scattered(const HCSR& A, const std::vector<int32_t>& iperm) {
 // down to kLeaf rows.  (One search over the whole graph gives fronts: on a
 // 200k-row torus graph a block of 1,316 consecutive rows then reads 4,900
 // rows, 3,100 with the pieces.)
-std::vector<int32_t> bisection_order(const HCSR& A) {
+std::vector<int32_t> bisection_order(const HCSR& A, int threads) {
   constexpr int64_t kLeaf = 1024;  // a window of the SELL copy
   const int64_t n = A.nrows;
   std::vector<int32_t> q(n), out(n), piece(n, 0);  // piece: the piece a row is in, fixed while pieces are searched
@@ -73,7 +73,7 @@ std::vector<int32_t> bisection_order(const HCSR& A) {
         piece[q[i]] = base + (int32_t)c;
         done[q[i]] = 0;
       }
-#pragma omp parallel for schedule(dynamic, 1)
+#pragma omp parallel for schedule(dynamic, 1) num_threads(threads)
     for (int64_t c = 0; c < (int64_t)cuts.size(); ++c) {
       const int64_t lo = cuts[c].lo, hi = cuts[c].hi;
       const int32_t id = base + (int32_t)c;

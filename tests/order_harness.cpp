@@ -9,14 +9,13 @@
 
 #include "order.h"
 
-static int g_team = 1;
 static std::atomic<long> g_dealt;
 static thread_local int t_id, t_team = 1;
 static thread_local long t_start, t_end, t_chunk;
 
 extern "C" {
 void GOMP_parallel(void (*fn)(void*), void* data, unsigned threads, unsigned) {
-  const int team = threads ? (int)threads : g_team;
+  const int team = (int)threads;
   g_dealt.store(0);
   auto run = [&](int id) {
     t_id = id;
@@ -77,12 +76,10 @@ int main() {
       const mmd::HCSR A = graph(n, far);
       std::vector<int32_t> own(n);
       for (int i = 0; i < n; ++i) own[i] = i;
-      g_team = 1;
-      const bool s = mmd::scattered(A, own);
-      const std::vector<int32_t> serial = mmd::bisection_order(A);
-      g_team = 6;
-      if (mmd::scattered(A, own) != s || s != (far > 0 && n > 1025)) return 1;
-      if (mmd::bisection_order(A) != serial) return 2;
+      const bool s = mmd::scattered(A, own, 1);
+      const std::vector<int32_t> serial = mmd::bisection_order(A, 1);
+      if (mmd::scattered(A, own, 6) != s || s != (far > 0 && n > 1025)) return 1;
+      if (mmd::bisection_order(A, 6) != serial) return 2;
       std::vector<char> seen(n, 0);
       for (int32_t r : serial) seen[r] = 1;
       for (char c : seen)
