@@ -547,3 +547,24 @@ def test_level_bsolve_deep(size):
         rounding = 9 * its * np.finfo(float).eps * abs(S).sum(1).max() * np.linalg.norm(xh)
         assert res <= tol * np.linalg.norm(b) + rounding
     h.close()
+
+
+@pytest.mark.parametrize("sigma,opts", [(0.1, {"loc_radius": 0, "s_max": 4}), (0.05, {}), (0.05, {"loc_radius": 0})])
+def test_level_op_ill_conditioned_mass(sigma, opts):
+    """OP on a level whose M^(1) is badly conditioned (1e4 to 1.6e5), down to 1e-13: the inner solves' recurrence.  The
+    residual that the outer recurrence carries meets the tolerance; the true one differs by the rounding of its updates."""
+    A = W.swissroll(1500, sigma=sigma)
+    h = _handle(A, n_coarse=20, **opts)
+    n = h.level_size(1)
+    L = h.level(1)  # the library's own matrices: phi of a nearly uncoupled patch is any of several
+    A1, M1 = (sp.csr_matrix((val, col, ptr), shape=(n, n)) for ptr, col, val in (L["A"], L["M"]))
+    x = np.random.default_rng(2).standard_normal(A1.shape[0])
+    b = M1 @ x
+    row = np.diff(A1.indptr).max()
+    for tol in (1e-11, 1e-12, 1e-13):
+        y = torch.zeros(len(x), dtype=torch.float64, device="cuda")
+        its = h.level_op(1, _dev(x), y, tol)
+        yh = y.cpu().numpy()
+        rounding = (row + 4) * its * np.finfo(float).eps * abs(A1).sum(1).max() * np.linalg.norm(yh)
+        assert np.linalg.norm(b - A1 @ yh) <= tol * np.linalg.norm(b) + rounding
+    h.close()
