@@ -4,11 +4,25 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "dev_common.cuh"
 
 namespace mmd {
+
+// Runs f at the first call for each device: a kernel's attributes belong to the
+// device that is current when they are set.
+struct PerDevice {
+  std::once_flag flag[64];
+  template <typename F>
+  void run(int device, F&& f) {
+    if (device < 0 || device >= 64)
+      f();
+    else
+      std::call_once(flag[device], f);
+  }
+};
 
 // SELL-32 view of a sparse matrix (see DCSR).
 struct Sell {

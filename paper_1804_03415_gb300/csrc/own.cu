@@ -31,7 +31,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "grid_comm.cuh"
@@ -421,10 +420,15 @@ __global__ void __launch_bounds__(kOwnThreads, 1) own_cg_kernel(SolverArgs a, Ow
   }
 }
 
+int current_device() {
+  int d = -1;
+  return cudaGetDevice(&d) == cudaSuccess ? d : -1;
+}
+
 template <bool CL>
 void own_attrs() {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice once;
+  once.run(current_device(), [] {
     cudaFuncSetAttribute(own_cg_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOwnSmem);
     if (CL) cudaFuncSetAttribute(own_cg_kernel<CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   });
@@ -437,8 +441,8 @@ bool near_fits(int64_t n) { return ((n + 31) / 32) * 8 <= kOwnSmem; }
 
 cudaError_t launch_near(const Sell& A, int64_t n, int grid, const int32_t* first, int stride, int32_t* count,
                         int32_t* list, uint16_t* lcol, cudaStream_t st) {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static PerDevice once;
+  once.run(current_device(), [] {
     cudaFuncSetAttribute(near_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOwnSmem);
   });
   near_kernel<<<grid, 1024, ((n + 31) / 32) * 8, st>>>(A, n, first, stride, count, list, lcol);

@@ -1,4 +1,5 @@
-// How a one-column launch of own.cu shares the rows and lays out its shared memory (host functions of the library).
+// How a one-column launch of own.cu shares the rows and lays out its shared memory, and prepares its kernels (host
+// functions of the library).
 #include <algorithm>
 #include <cstdio>
 
@@ -46,6 +47,16 @@ int main() {
   // shares stay even up to the largest offsets that 32 bits hold
   const std::vector<int32_t> wide = offsets(60, 1100000), first = mmd::own_shares(wide.data(), 60, 16);
   for (int b = 0; b < 16; ++b) CHECK(first[b + 1] - first[b] >= 3 && first[b + 1] - first[b] <= 5);
+  // once for each device
+  mmd::PerDevice once;
+  int runs[64] = {}, beyond = 0;
+  for (int i = 0; i < 3; ++i) {
+    for (int d = 0; d < 64; ++d) once.run(d, [&] { ++runs[d]; });
+    once.run(64, [&] { ++beyond; });
+    once.run(-1, [&] { ++beyond; });
+  }
+  for (int d = 0; d < 64; ++d) CHECK(runs[d] == 1);
+  CHECK(beyond == 6);
   std::puts("plans hold");
   return 0;
 }
