@@ -94,3 +94,58 @@ def test_own_cg_cluster_sizes(blocks):
         nb = np.linalg.norm(b)
         assert np.linalg.norm(b - A @ x) <= 2 * TOL * nb
         assert np.linalg.norm(x - spl.spsolve(A.tocsc(), b)) <= 2 * TOL * nb
+
+
+def kernels_of(call):
+    """Names of the kernels that a call launches; skips where the tracer gives none."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    names = set()
+    for _ in range(3):  # the first trace of a process may hold nothing
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            call()
+            torch.cuda.synchronize()
+        names |= {e.key for e in p.key_averages()}
+    if not any("kernel" in s for s in names):
+        pytest.skip("no kernel records on this machine")
+    return names
+
+
+@pytest.mark.parametrize("kind,n,kernel", [
+    ("path", 33, "own_cg_kernel<true>"), ("rand", 3000, "own_cg_kernel<true>"), ("rand", 9000, "own_cg_kernel<false>"),
+    ("path", 200000, "own_cg_kernel<false>"), ("hub", 20000, "solve_kernel<1, double, 0>"),
+    ("path", 600000, "solve_kernel<1, double, 0>")])
+def test_which_kernel(kind, n, kernel):
+    import torch
+
+    import paper_1804_03415_gb300 as G
+
+    A = sp.csr_matrix(matrix(kind, n))
+    A.sort_indices()
+    h = G.MMD(A.indptr.astype(np.int32), A.indices.astype(np.int32), A.data, k_max=0)
+    x = torch.ones(n, dtype=torch.float64, device="cuda")
+    y = torch.zeros_like(x)
+    ran = kernels_of(lambda: h.level_op(0, x, y, TOL))
+    assert any(kernel in s for s in ran), ran
+    assert sum("own_cg" in s or "solve_kernel" in s for s in ran) == 1, ran
+    h.close()
+
+
+@pytest.mark.parametrize("n", [400, 6000])
+def test_wait_runs_out_then_recovers(n):
+    """Lanczos with plain CG on a handle without levels: its first device waits are those of the one-column launch, on a
+    cluster and on a grid.  They give up after the limit, the call says so, and the handle solves on."""
+    import workloads as W
+
+    import paper_1804_03415_gb300 as G
+
+    A = W.random_spd_mmatrix(n, 6, seed=9, shift=0.5)
+    h = G.MMD(A.rowptr, A.col, A.val, k_max=0)
+    for _ in range(2):
+        with pytest.raises(G.MMDError) as ei:
+            h.eig_leftmost(4, 1e-8, method=G.MMD_IRLM_CG, timeout_s=1e-9)
+        assert ei.value.code == G._lib.MMD_ETIMEOUT
+        lam, V, st = h.eig_leftmost(4, 1e-8, method=G.MMD_IRLM_CG)
+        assert st["max_rel_residual"] <= 10 * 1e-8
+    h.close()
