@@ -62,10 +62,12 @@ PRECISIONS = {"fp64": 0, "mixed": 1, "mixed_all": 2}  # MMD_FP64, MMD_MIXED, MMD
 FP64_FMA_PER_CLK_SM = 1.68
 FP64_PEAK_TFLOPS = 152 * FP64_FMA_PER_CLK_SM * 2 * 2.070e9 / 1e12  # 1.057
 FP64_NOMINAL_TFLOPS = 1.25
-# DRAM bytes (read + write) per launch of the level-0 Operator OP kernel, solve_kernel<1, double, 0>,
-# from the ncu capture summarised in profiles/solve_kernel_op_torus_knn_200k_level0.md (32.63 MB read +
-# 0.81 MB written: the 30 MB level-0 matrix and the vectors once, every iteration after the first from L2)
-TRAFFIC_PER_LAUNCH = 33.44e6
+# DRAM bytes (read + write) per launch of the FP64 level-0 Operator OP kernel, own_cg_kernel<false>,
+# from the ncu capture summarised in profiles/own_cg_kernel_op_torus_knn_200k.md (29.07 MB read + 0.48 MB
+# written: the level-0 matrix once, every iteration after the first from shared memory and L2)
+TRAFFIC_PER_LAUNCH = 29.55e6
+# the kernel of the level-0 Operator OP (CG on A, one column) in each precision
+OP_KERNEL = {"fp64": "own_cg_kernel<false>", "mixed": "dd_cg_kernel<1>", "mixed_all": "solve_kernel<1, float, 0>"}
 REF_EIGS = os.path.join(ROOT, "tests", "golden", "torus_knn_200k_eigs.json")
 
 
@@ -364,24 +366,24 @@ def gpu_arm(args, rank, world):
         "e2e": {"value": world * N / e2e_s, "unit": "eigenpairs/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "includes": "mmd_build from host CSR + eig_leftmost to host, one run"},
         "gpu_launches": int(sum(s["kernel_launches"] for s in stats)),
-        "roofline": {"kernel": "solve_kernel<1, double, 0> (level-0 Operator OP: CG on A, one column)",
+        "roofline": {"kernel": OP_KERNEL[args.precision] + " (level-0 Operator OP: CG on A, one column)",
                      "bound": "alu", "achieved": op_tflops, "peak": FP64_PEAK_TFLOPS,
                      "peak_source": "derived: 152 SMs x 1.68 FP64 FMA/clk/SM (measured on one SM) x 2 x 2.07 GHz; "
                                     f"nominal {FP64_NOMINAL_TFLOPS}",
                      "unit": "TFLOP/s", "frac": (op_tflops / FP64_PEAK_TFLOPS) if op_tflops else None,
                      "traffic": TRAFFIC_PER_LAUNCH if args.precision == "fp64" else None,
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch "
-                                       "(profiles/solve_kernel_op_torus_knn_200k_level0.md)",
+                                       "(profiles/own_cg_kernel_op_torus_knn_200k.md)",
                      "launches": op_launches, "iterations": op_iters,
                      "algorithmic_flops_per_launch": (op_flops / op_launches) if op_launches else None,
                      "share_of_step": op_ms / max(ms_local, 1e-9),
-                     "note": "latency bound (grid barriers, reduction rounds, L2 gathers of the SpMV): the 30 MB "
-                             "level-0 matrix stays in L2 across iterations; algorithmic flops per iteration "
-                             "2 nnz(A) + 10 n",
+                     "note": "FP64 issue and the exchange of an iteration (one grid-wide sum, the fetch of the rows "
+                             "that a block reads): three quarters of the matrix stay in shared memory, the rest is "
+                             "streamed from L2; algorithmic flops per iteration 2 nnz(A) + 10 n",
                      "hbm_view": {"achieved": op_gbs, "peak": peak, "peak_source": src, "unit": "GB/s",
                                   "frac": (op_gbs / peak) if op_gbs else None,
                                   "bytes": "12 nnz + 4 n per iteration (matrix) + 72 n (vectors)"}},
-        "solver_all": {"kernel": "solve_kernel, every instance (OP, refinement tiles, coarse levels)",
+        "solver_all": {"kernel": "every solver launch (OP, refinement tiles, coarse levels)",
                        "achieved_tflops": tflops, "frac_of_fp64_peak": (tflops / FP64_PEAK_TFLOPS) if tflops else None,
                        "achieved_gbs": gbs, "launches": pcg_launches, "share_of_step": pcg_ms / max(ms_local, 1e-9),
                        "note": "the refinement's tiles run on four concurrent lanes, so their event-timed "
