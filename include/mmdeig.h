@@ -327,7 +327,9 @@ int mmd_spmv_tuning(const mmd_handle* h, int k, int which, float* ms_per_variant
  * 20 iterations of CG on A^(k) at each of MMD_TUNE_GRIDS candidate grids
  * (2 ... 152 blocks of 1024 threads, those that are resident and leave at
  * least 64 rows per block) and runs that level's solves on the fastest grid
- * (capped by the SMs a batched call or a concurrent tile lane may use).
+ * (capped by the SMs a batched call or a concurrent tile lane may use).  FP64
+ * CG on A^(k) for one right-hand side does not use the choice for mt = 1 where
+ * its own kernel runs it, which takes its grid from the matrix.
  * Returns the chosen grid, writes the candidates to grids and their measured
  * microseconds per iteration to us_per_iter (0 = not tried) unless NULL;
  * MMD_EINVAL for a host-only handle, k outside [0, K) or mt not 1 / 4.  The

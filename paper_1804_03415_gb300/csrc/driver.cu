@@ -1618,7 +1618,9 @@ int level_op_block(mmd_handle* h, int k, int m, const double* x, double* y, doub
 // right-hand side (tolerance out of reach, so every trial runs the same
 // iterations) are timed with events at each candidate grid that is resident
 // and leaves at least 64 rows per block; the fastest grid is kept in the
-// level.  Runs once per handle, on a private stream, before any solve.
+// level.  The trials are solve_kernel's (plain_cg), which runs every preconditioned
+// and multi-column solve of the level; one column of FP64 CG goes through own.cu
+// on a grid of its own (own_choice) where that launch fits.  Runs once per handle, on a private stream, before any solve.
 int tune_solver(mmd_handle* h) {
   cudaStream_t st = nullptr;
   try {

@@ -18,9 +18,11 @@
 // themselves.  The block's part of the matrix is staged in shared memory, as
 // many slices as fit, the rest is streamed from L2.
 //
-// Measured, cycles per iteration at 2.07 GHz, before -> after (solve_kernel
-// on the same matrices): 64 x 64 grid operator 19.6k -> 9.3k; geometric graph
-// of 50k rows 37k -> 20k; point-cloud graph of 200k rows 98k -> 55k.
+// Measured, us an iteration, solve_kernel on the rows as they came -> here:
+// 64 x 64 operator 9.7 -> 4.6, 256 x 256 12.0 -> 6.7; 10-nearest-neighbour
+// graphs of 2k rows 10.5 -> 5.3, 20k 14.5 -> 7.1, 50k 15.5 -> 8.2, 200k 20.5 ->
+// 15.3 (17.8 before in the order of a handle's patches); geometric graph of 100k
+// rows 16.0 -> 9.2.  Where it would lose: own_plan.
 //
 // Two instances:
 //   grid     a cooperative launch over many SMs, sums and barriers of
